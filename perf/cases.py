@@ -70,7 +70,7 @@ def draw(rng):
     prec = "f64" if rng.random() < 0.15 else "f32"
     top = {"gradient": 8, "graph": 7, "forward": 8, "power": 9, "ic": 9}.get(kind, 10)
     if prec == "f64":
-        top = min(top, 8)
+        top = min(top, 7 if kind in RUN_KINDS else 8)
     lg = rng.randint(5, top)
     if lg == 10 and rng.random() < 0.5:
         lg = 9
