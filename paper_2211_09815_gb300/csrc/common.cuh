@@ -6,6 +6,8 @@
 
 namespace pmgb {
 
+constexpr int kNumSms = 152;   // SMs of a GB300
+
 template <typename T> struct Cx;
 template <> struct Cx<float> { using type = float2; };
 template <> struct Cx<double> { using type = double2; };

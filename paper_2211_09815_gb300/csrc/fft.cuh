@@ -218,26 +218,35 @@ __device__ __forceinline__ void fft_tile(const Src& src, const Mid& mid, const D
   }
 }
 
-// Tile shapes.  Column passes: TC sequences of length L in one tile of <= BYTES,
+// Tile shapes.  Column passes: TC sequences of length L in one tile of <= 64 KB,
 // NT = TC * L / RMAX threads (each thread holds RMAX values), NT <= 512.
-template <typename T, int L, int BYTES = 65536> struct ColTile {
+//
+// SM (small): tiles of about 64 threads.  A pass over few sequences -- a side plane, a mesh
+// or a lattice of 64^3 and below -- makes fewer full tiles than there are SMs, and most of
+// the chip idles; the small tiles spread it (small_tiles).  Every thread does the same work
+// in both.  Measured (full -> small tiles, main and side columns in one launch): FP64
+// forward run of 10 steps on 64^3 4.16 -> 1.59 ms (its 64^3 passes ran on 32 SMs), FP32
+// force on 128^3 195 -> 160 us (its side planes ran on 2 to 8 SMs).
+template <typename T, int L, bool SM = false> struct ColTile {
   static constexpr int RMAX = Plan<L>::RMAX;
-  static constexpr int TC0 = BYTES / (L * (int)sizeof(cx_t<T>));
+  static constexpr int TC0 = 65536 / (L * (int)sizeof(cx_t<T>));
   static constexpr int TC1 = TC0 > 256 ? 256 : TC0;
   static constexpr int TCMAXNT = 512 * RMAX / L;
   static constexpr int TC2 = TC1 < TCMAXNT ? TC1 : TCMAXNT;
-  static constexpr int TC = TC2 < 1 ? 1 : TC2;
+  static constexpr int TCF = TC2 < 1 ? 1 : TC2;
+  // at least four sequences, so that the runs of a strided pass fill a 32-byte sector
+  static constexpr int TCS0 = 64 * RMAX / L < 4 ? 4 : 64 * RMAX / L;
+  static constexpr int TC = SM && TCS0 < TCF ? TCS0 : TCF;
   static constexpr int NT = TC * L / RMAX;
   static constexpr int LD = TC;
   static constexpr int SMEM = skew_rows(L) * LD * (int)sizeof(cx_t<T>);
 };
-// Fused z passes keep two tiles of the column-pass shape.
-template <typename T, int L> using FusedTile = ColTile<T, L, 65536>;
 // Row passes (x axis): TR rows of L = n/2 complex values, tile padded to LD = TR + 1 so
 // that the transposing row loads do not collide in shared-memory banks.  Rows of 512
 // points run the two-stage radix-32 plan on 64 KB tiles (one shared-memory round trip less
-// than three radix-8 stages); shorter rows the three-stage plans on 32 KB tiles.
-template <typename T, int L> struct RowTile {
+// than three radix-8 stages); shorter rows the three-stage plans on 32 KB tiles.  SM: small
+// tiles for meshes of few rows, as above.
+template <typename T, int L, bool SM = false> struct RowTile {
   using P = Plan2<L>;
   static constexpr int RMAX = P::RMAX;
   static constexpr int TR0 = (RMAX == 32 ? 65536 : 32768) / (L * (int)sizeof(cx_t<T>));
@@ -246,7 +255,9 @@ template <typename T, int L> struct RowTile {
   static constexpr int TR2 = TR1 < TRMAXNT ? TR1 : TRMAXNT;
   // a tile never spans two instances: TR divides the n^2 = 4 L^2 rows of one mesh
   static constexpr int TR3 = TR2 < 4 * L * L ? TR2 : 4 * L * L;
-  static constexpr int TR = TR3 < 1 ? 1 : TR3;
+  static constexpr int TRF = TR3 < 1 ? 1 : TR3;
+  static constexpr int TRS0 = 64 * RMAX / L < 4 ? 4 : 64 * RMAX / L;
+  static constexpr int TR = SM && TRS0 < TRF ? TRS0 : TRF;
   // at most 256 threads (measured faster than one radix item per thread at L = 512)
   static constexpr int NT0 = TR * L / RMAX;
   static constexpr int NT = NT0 > 256 ? 256 : NT0;
@@ -254,5 +265,7 @@ template <typename T, int L> struct RowTile {
   static constexpr int LD = TR + 1;
   static constexpr int SMEM = skew_rows(L) * LD * (int)sizeof(cx_t<T>);
 };
+// whether a pass of `tiles` full tiles takes the small ones: below two tiles per SM
+inline bool small_tiles(long long tiles) { return tiles < 2 * kNumSms; }
 
 }  // namespace pmgb

@@ -23,15 +23,15 @@ __device__ __forceinline__ long long seq_base(const SeqMap& m, int s) {
   const int t = s / m.ncols;
   const int o0 = t % m.n0;
   const int o1 = t / m.n0;
-  return (long long)o1 * m.os1 + (long long)o0 * m.os0 + (long long)col * m.cs;
+  return m.off + (long long)o1 * m.os1 + (long long)o0 * m.os0 + (long long)col * m.cs;
 }
 
-template <typename T, int L, int DIR>
-__global__ void __launch_bounds__(ColTile<T, L>::NT, 2)
+template <typename T, int L, int DIR, bool SM>
+__global__ void __launch_bounds__(ColTile<T, L, SM>::NT, SM ? 1 : 2)
 k_fft_cols(const SeqMap mm, const SeqMap ms, int ntiles_main, ColBufs<T> bufs,
            const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
-  using TL = ColTile<T, L>;
+  using TL = ColTile<T, L, SM>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
   const bool side = blockIdx.x >= (unsigned)ntiles_main;
@@ -83,12 +83,12 @@ struct GMergeIK {    // out = A + i k2 v
   }
 };
 
-template <typename T, int L, int MODE>   // MODE 1: split, 2: merge
-__global__ void __launch_bounds__(ColTile<T, L>::NT, 1)
+template <typename T, int L, int MODE, bool SM>   // MODE 1: split, 2: merge
+__global__ void __launch_bounds__(ColTile<T, L, SM>::NT, 1)
 k_fft_cols_yx(const SeqMap mm, const SeqMap ms, int ntiles_main, ColBufs<T> bufs,
               const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
-  using TL = ColTile<T, L>;
+  using TL = ColTile<T, L, SM>;
   constexpr int TILE = skew_rows(L) * TL::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* A = reinterpret_cast<C*>(smem_raw);
@@ -128,12 +128,12 @@ k_fft_cols_yx(const SeqMap mm, const SeqMap ms, int ntiles_main, ColBufs<T> bufs
 // (k, L - k), k < L/2, of every row, indexed row-major so that a power of two divides them,
 // and then the middle k = L/2 of every row; the address of each row of the tile is worked
 // out once, into shared memory.
-template <typename T, int L>
-__global__ void __launch_bounds__(RowTile<T, L>::NT)
+template <typename T, int L, bool SM>
+__global__ void __launch_bounds__(RowTile<T, L, SM>::NT)
 k_fft_x_r2c(RowJob<T> job, int nrows, int nbuf, const cx_t<T>* __restrict__ twL,
             const cx_t<T>* __restrict__ twN) {
   using C = cx_t<T>;
-  using TL = RowTile<T, L>;
+  using TL = RowTile<T, L, SM>;
   constexpr int N = 2 * L;
   constexpr int RT = TL::TR;   // rows per tile
   constexpr int KH = L / 2;
@@ -213,11 +213,11 @@ struct C2RUntangle {
   __device__ __forceinline__ static int freq(int u) { return u < PAIRS ? u % KH : KH; }
 };
 
-template <typename T, int L>
-__global__ void __launch_bounds__(RowTile<T, L>::NT)
+template <typename T, int L, bool SM>
+__global__ void __launch_bounds__(RowTile<T, L, SM>::NT)
 k_fft_x_c2r(RowJob<T> job, int nrows, const cx_t<T>* __restrict__ twL, const cx_t<T>* __restrict__ twN) {
   using C = cx_t<T>;
-  using TL = RowTile<T, L>;
+  using TL = RowTile<T, L, SM>;
   using U = C2RUntangle<T, L, TL::TR, TL::NT>;
   constexpr int N = 2 * L;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -287,9 +287,9 @@ k_fft_x_c2r(RowJob<T> job, int nrows, const cx_t<T>* __restrict__ twL, const cx_
 // instances back to back) so that a gather reads all components of a corner with one
 // load.  The block holds TR/4 rows of each component; a null spectrum pointer reads as 0.
 // Component dq (or none if dq < 0) is multiplied by -i k_x on the way in.
-template <typename T, int L, int Q> struct C2R4Tile {
+template <typename T, int L, int Q, bool SM = false> struct C2R4Tile {
   using P = typename RowTile<T, L>::P;
-  static constexpr int RT = RowTile<T, L>::TR / 4;       // rows per block
+  static constexpr int RT = RowTile<T, L, SM>::TR / 4;   // rows per block
   static constexpr int TR = Q * RT;                      // sequences per block
   // above 256 threads, two radix items per thread (measured faster at L = 512)
   static constexpr int NT0 = TR * L / P::RMAX;
@@ -302,12 +302,12 @@ template <typename T, int L, int Q> struct C2R4Tile {
 // field of a row scaled by 2^-e so that the row's largest magnitude lies in [2^14, 2^15),
 // e stored as one int8 per (row, field) in fexp ([rows][4]); FP16 keeps 11 significant
 // bits of every value in the row down to 2^-29 of its largest.
-template <typename T, int L, int Q, bool H = false>
-__global__ void __launch_bounds__(C2R4Tile<T, L, Q>::NT)
+template <typename T, int L, int Q, bool SM, bool H>
+__global__ void __launch_bounds__(C2R4Tile<T, L, Q, SM>::NT)
 k_fft_x_c2r4(RowJob<T> job, int nrows, int dq, void* __restrict__ out, signed char* __restrict__ fexp,
              const cx_t<T>* __restrict__ twL, const cx_t<T>* __restrict__ twN) {
   using C = cx_t<T>;
-  using TL = C2R4Tile<T, L, Q>;
+  using TL = C2R4Tile<T, L, Q, SM>;
   using U = C2RUntangle<T, L, TL::TR, TL::NT>;
   constexpr int N = 2 * L;
   constexpr int RT = TL::RT;
@@ -543,11 +543,11 @@ __device__ __forceinline__ GreenSeq<T> green_seq(const ZSeq& q, const T* coef, c
 }
 
 // Forward force: delta^ (after x, y) --z FFT--> * (-i k_0 G), * G --z IFFT--> z force, U
-template <typename T, int L>
-__global__ void __launch_bounds__(FusedTile<T, L>::NT)
+template <typename T, int L, bool SM>
+__global__ void __launch_bounds__(ColTile<T, L, SM>::NT)
 k_fused_z_force(ZJob<T> job, int ntiles_main, const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
-  using TL = FusedTile<T, L>;
+  using TL = ColTile<T, L, SM>;
   constexpr int TILE = skew_rows(L) * TL::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* A = reinterpret_cast<C*>(smem_raw);
@@ -572,11 +572,11 @@ k_fused_z_force(ZJob<T> job, int ntiles_main, const cx_t<T>* __restrict__ tw) {
 
 // Adjoint: P_0, V = i (k_1 P_1 + k_2 P_2) (after x, y) --z FFT--> G (i k_0 P_0 + V)
 // --z IFFT--> psi
-template <typename T, int L>
-__global__ void __launch_bounds__(FusedTile<T, L>::NT)
+template <typename T, int L, bool SM>
+__global__ void __launch_bounds__(ColTile<T, L, SM>::NT)
 k_fused_z_adjoint(ZJob<T> job, int ntiles_main, const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
-  using TL = FusedTile<T, L>;
+  using TL = ColTile<T, L, SM>;
   constexpr int TILE = skew_rows(L) * TL::LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* A = reinterpret_cast<C*>(smem_raw);
@@ -605,66 +605,106 @@ static void set_smem(const void* fn, size_t bytes) {
   if (bytes > 48 * 1024) ensure_smem_attr(fn, (int)bytes);
 }
 
-template <typename T, int L, int DIR>
-static void launch_cols_L(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, int nbuf,
+// tiles of TC sequences for nseq sequences
+inline int tiles_for(int nseq, int tc) { return nseq > 0 ? (nseq + tc - 1) / tc : 0; }
+
+template <typename T, int L, int DIR, bool SM>
+static void launch_cols_S(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, int nbuf,
                           const cx_t<T>* tw, cudaStream_t st) {
-  using TL = ColTile<T, L>;
-  const int ntm = (mm.nseq + TL::TC - 1) / TL::TC;
-  const int nts = ms.nseq > 0 ? (ms.nseq + TL::TC - 1) / TL::TC : 0;
+  using TL = ColTile<T, L, SM>;
+  const int ntm = tiles_for(mm.nseq, TL::TC), nts = tiles_for(ms.nseq, TL::TC);
   const size_t sm = TL::SMEM;
-  auto fn = k_fft_cols<T, L, DIR>;
+  auto fn = k_fft_cols<T, L, DIR, SM>;
   set_smem<T, L>((const void*)fn, sm);
   dim3 grid(ntm + nts, nbuf);
   fn<<<grid, TL::NT, sm, st>>>(mm, ms, ntm, bufs, tw + L);
 }
+template <typename T, int L, int DIR>
+static void launch_cols_L(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, int nbuf,
+                          const cx_t<T>* tw, cudaStream_t st) {
+  if (small_tiles((long long)nbuf * tiles_for(mm.nseq + ms.nseq, ColTile<T, L>::TC)))
+    launch_cols_S<T, L, DIR, true>(mm, ms, bufs, nbuf, tw, st);
+  else
+    launch_cols_S<T, L, DIR, false>(mm, ms, bufs, nbuf, tw, st);
+}
 
-template <typename T, int L, int MODE>
-static void launch_cols_yx_L(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, const cx_t<T>* tw,
+template <typename T, int L, int MODE, bool SM>
+static void launch_cols_yx_S(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, const cx_t<T>* tw,
                              cudaStream_t st) {
-  using TL = ColTile<T, L>;
-  const int ntm = (mm.nseq + TL::TC - 1) / TL::TC;
-  const int nts = ms.nseq > 0 ? (ms.nseq + TL::TC - 1) / TL::TC : 0;
+  using TL = ColTile<T, L, SM>;
+  const int ntm = tiles_for(mm.nseq, TL::TC), nts = tiles_for(ms.nseq, TL::TC);
   const size_t sm = 2 * (size_t)TL::SMEM;
-  auto fn = k_fft_cols_yx<T, L, MODE>;
+  auto fn = k_fft_cols_yx<T, L, MODE, SM>;
   set_smem<T, L>((const void*)fn, sm);
   fn<<<ntm + nts, TL::NT, sm, st>>>(mm, ms, ntm, bufs, tw + L);
 }
+template <typename T, int L, int MODE>
+static void launch_cols_yx_L(const SeqMap& mm, const SeqMap& ms, const ColBufs<T>& bufs, const cx_t<T>* tw,
+                             cudaStream_t st) {
+  if (small_tiles(tiles_for(mm.nseq + ms.nseq, ColTile<T, L>::TC)))
+    launch_cols_yx_S<T, L, MODE, true>(mm, ms, bufs, tw, st);
+  else
+    launch_cols_yx_S<T, L, MODE, false>(mm, ms, bufs, tw, st);
+}
 
-template <typename T, int L>
-static void launch_r2c_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
-  using TL = RowTile<T, L>;
+template <typename T, int L, bool SM>
+static void launch_r2c_S(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
+  using TL = RowTile<T, L, SM>;
   const size_t sm = TL::SMEM;
-  dim3 grid(((nrows + TL::TR - 1) / TL::TR) * nbuf, 1);
-  auto fn = k_fft_x_r2c<T, L>;
+  dim3 grid(tiles_for(nrows, TL::TR) * nbuf, 1);
+  auto fn = k_fft_x_r2c<T, L, SM>;
   set_smem<T, L>((const void*)fn, sm);
   fn<<<grid, TL::NT, sm, st>>>(job, nrows, nbuf, tw + L, tw + 2 * L);
 }
-
 template <typename T, int L>
-static void launch_c2r_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
-  using TL = RowTile<T, L>;
+static void launch_r2c_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
+  if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
+    launch_r2c_S<T, L, true>(job, nbuf, nrows, tw, st);
+  else
+    launch_r2c_S<T, L, false>(job, nbuf, nrows, tw, st);
+}
+
+template <typename T, int L, bool SM>
+static void launch_c2r_S(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
+  using TL = RowTile<T, L, SM>;
   const size_t sm = TL::SMEM;
-  dim3 grid((nrows + TL::TR - 1) / TL::TR, nbuf);
-  auto fn = k_fft_x_c2r<T, L>;
+  dim3 grid(tiles_for(nrows, TL::TR), nbuf);
+  auto fn = k_fft_x_c2r<T, L, SM>;
   set_smem<T, L>((const void*)fn, sm);
   fn<<<grid, TL::NT, sm, st>>>(job, nrows, tw + L, tw + 2 * L);
 }
-
 template <typename T, int L>
-static void launch_fused_L(const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st) {
-  using TL = FusedTile<T, L>;
-  const int ntm = (job.batch * L * (L / 2) + TL::TC - 1) / TL::TC;
-  const int nts = (job.batch * L + TL::TC - 1) / TL::TC;
+static void launch_c2r_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
+  if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
+    launch_c2r_S<T, L, true>(job, nbuf, nrows, tw, st);
+  else
+    launch_c2r_S<T, L, false>(job, nbuf, nrows, tw, st);
+}
+
+// fused z pass of the main columns (main = 0: of the side plane alone)
+template <typename T, int L, bool SM>
+static void launch_fused_S(const ZJob<T>& job, bool adjoint, bool main, const cx_t<T>* tw, cudaStream_t st) {
+  using TL = ColTile<T, L, SM>;
+  const int ntm = main ? tiles_for(job.batch * L * (L / 2), TL::TC) : 0;
+  const int nts = tiles_for(job.batch * L, TL::TC);
   const size_t sm = 2 * (size_t)TL::SMEM;
   if (adjoint) {
-    auto fn = k_fused_z_adjoint<T, L>;
+    auto fn = k_fused_z_adjoint<T, L, SM>;
     set_smem<T, L>((const void*)fn, sm);
     fn<<<ntm + nts, TL::NT, sm, st>>>(job, ntm, tw + L);
   } else {
-    auto fn = k_fused_z_force<T, L>;
+    auto fn = k_fused_z_force<T, L, SM>;
     set_smem<T, L>((const void*)fn, sm);
     fn<<<ntm + nts, TL::NT, sm, st>>>(job, ntm, tw + L);
   }
+}
+template <typename T, int L>
+static void launch_fused_L(const ZJob<T>& job, bool adjoint, bool main, const cx_t<T>* tw, cudaStream_t st) {
+  const int nseq = job.batch * L * (main ? L / 2 + 1 : 1);
+  if (small_tiles(tiles_for(nseq, ColTile<T, L>::TC)))
+    launch_fused_S<T, L, true>(job, adjoint, main, tw, st);
+  else
+    launch_fused_S<T, L, false>(job, adjoint, main, tw, st);
 }
 
 template <typename T, int L> static int tiles_of() { return L * ((L / 2) / TmaTile<T, L>::TC); }
@@ -859,17 +899,26 @@ int fft_x_r2c(int n, const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* t
   return PM_OK;
 }
 
+template <typename T, int L, int Q, bool SM>
+static void launch_c2r4_S(const RowJob<T>& job, int nrows, int dq, void* out, signed char* fexp, const cx_t<T>* tw,
+                          cudaStream_t st) {
+  using TL = C2R4Tile<T, L, Q, SM>;
+  const size_t sm = TL::SMEM;
+  auto fn = k_fft_x_c2r4<T, L, Q, SM, false>;
+  if constexpr (sizeof(T) == 4)
+    if (fexp) fn = k_fft_x_c2r4<T, L, Q, SM, true>;
+  set_smem<T, L>((const void*)fn, sm);
+  fn<<<tiles_for(nrows, TL::RT), TL::NT, sm, st>>>(job, nrows, dq, out, fexp, tw + L, tw + 2 * L);
+}
 template <typename T, int L, int Q>
 static void launch_c2r4_LQ(const RowJob<T>& job, int nrows, int dq, void* out, signed char* fexp, const cx_t<T>* tw,
                            cudaStream_t st) {
   using TL = C2R4Tile<T, L, Q>;
   if constexpr (RowTile<T, L>::TR % 4 == 0 && (TL::TR * L) % TL::P::RMAX == 0) {
-    const size_t sm = TL::SMEM;
-    auto fn = k_fft_x_c2r4<T, L, Q, false>;
-    if constexpr (sizeof(T) == 4)
-      if (fexp) fn = k_fft_x_c2r4<T, L, Q, true>;
-    set_smem<T, L>((const void*)fn, sm);
-    fn<<<(nrows + TL::RT - 1) / TL::RT, TL::NT, sm, st>>>(job, nrows, dq, out, fexp, tw + L, tw + 2 * L);
+    if (small_tiles(tiles_for(nrows, TL::RT)))
+      launch_c2r4_S<T, L, Q, true>(job, nrows, dq, out, fexp, tw, st);
+    else
+      launch_c2r4_S<T, L, Q, false>(job, nrows, dq, out, fexp, tw, st);
   }
 }
 template <typename T, int L>
@@ -895,33 +944,10 @@ int fft_x_c2r(int n, const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* t
   return PM_OK;
 }
 
-template <typename T, int L>
-static void launch_fused_side_L(const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st) {
-  using TL = FusedTile<T, L>;
-  const int nts = (job.batch * L + TL::TC - 1) / TL::TC;
-  const size_t sm = 2 * (size_t)TL::SMEM;
-  if (adjoint) {
-    auto fn = k_fused_z_adjoint<T, L>;
-    set_smem<T, L>((const void*)fn, sm);
-    fn<<<nts, TL::NT, sm, st>>>(job, 0, tw + L);
-  } else {
-    auto fn = k_fused_z_force<T, L>;
-    set_smem<T, L>((const void*)fn, sm);
-    fn<<<nts, TL::NT, sm, st>>>(job, 0, tw + L);
-  }
-}
-
 template <typename T>
-int fft_fused_side(int n, const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st) {
+int fft_fused_z(int n, const ZJob<T>& job, bool adjoint, bool main, const cx_t<T>* tw, cudaStream_t st) {
   if (n < 4) return PM_ERR_ARG;
-  PMGB_DISPATCH_L(n, (launch_fused_side_L<T, (LL < 4 ? 4 : LL)>(job, adjoint, tw, st)));
-  return PM_OK;
-}
-
-template <typename T>
-int fft_fused_z(int n, const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st) {
-  if (n < 4) return PM_ERR_ARG;
-  PMGB_DISPATCH_L(n, (launch_fused_L<T, (LL < 4 ? 4 : LL)>(job, adjoint, tw, st)));
+  PMGB_DISPATCH_L(n, (launch_fused_L<T, (LL < 4 ? 4 : LL)>(job, adjoint, main, tw, st)));
   return PM_OK;
 }
 

@@ -220,7 +220,7 @@ class Engine : public EngineBase {
   // ------------------------------------------------------------------ forward
   int forward(void* disp, void* mom, void* dens) override {
     counted_ = false;
-    prof_.begin(st_, P_OTHER, lpt2_ ? 12 + 26 : 12);
+    prof_.begin(st_, P_OTHER, lpt2_ ? 8 + 18 : 8);
     PMGB_RET(initial_conditions());
     prof_.end(st_, P_OTHER);
     for (int j = 0; j <= n_; ++j) {
@@ -364,7 +364,7 @@ class Engine : public EngineBase {
       }
     }
     // per-step sums: part_[(2j+q)][b][G] -> steps_[(2j+q)][b]
-    prof_.begin(st_, P_OTHER, lpt2_ ? 16 + 39 : 16);
+    prof_.begin(st_, P_OTHER, lpt2_ ? 12 + 27 : 12);
     k_sum_partials<<<2 * (n_ + 1) * B_, 256, 0, st_>>>(part_, G_, steps_, 1.0);
     PMGB_CK(cudaGetLastError());
     PMGB_RET(ic_adjoint(djdw));
@@ -865,19 +865,17 @@ class Engine : public EngineBase {
 
   // ---------------------------------------------------------------- FFT helpers
   SeqMap ymap(int n) const {
-    return SeqMap{n / 2, 1, n / 2, (long long)n * (n / 2), n, spec_len_cx(n), B_ * n * (n / 2)};
+    return SeqMap{n / 2, 1, n / 2, (long long)n * (n / 2), n, spec_len_cx(n), B_ * n * (n / 2), 0};
   }
   SeqMap yside(int n) const {
-    return SeqMap{1, n, n, spec_len_cx(n), B_, 0, B_ * n};
+    return SeqMap{1, n, n, spec_len_cx(n), B_, 0, B_ * n, spec_main_len(n)};
   }
   SeqMap zmap(int n) const {
-    return SeqMap{(long long)n * (n / 2), 1, n / 2, n / 2, n, spec_len_cx(n), B_ * n * (n / 2)};
+    return SeqMap{(long long)n * (n / 2), 1, n / 2, n / 2, n, spec_len_cx(n), B_ * n * (n / 2), 0};
   }
   SeqMap zside(int n) const {
-    return SeqMap{n, 1, n, spec_len_cx(n), B_, 0, B_ * n};
+    return SeqMap{n, 1, n, spec_len_cx(n), B_, 0, B_ * n, spec_main_len(n)};
   }
-  // column pass over up to 4 buffers (main + side planes); side maps are offset by the
-  // main length through the buffer pointers
   int spec_index(const C* p) const {
     for (int q = 0; q < 7; ++q)
       if (spec_[q] == p) return q;
@@ -886,6 +884,8 @@ class Engine : public EngineBase {
   // column pass over up to 4 spectra: mesh spectra (z-blocked main rows at 1024^3, see
   // spec_row) take the TMA-staged passes, lattice spectra (plain order) the unstaged ones
   int cols(int n, int dir, bool zaxis, C* const* bufs, int nb, bool mesh = true) {
+    SeqMap mm = zaxis ? zmap(n) : ymap(n);
+    const SeqMap ms = zaxis ? zside(n) : yside(n);
     if (use_tma_ && mesh && n == nm_) {
       CUtensorMap maps[4];
       for (int q = 0; q < nb; ++q) {
@@ -895,26 +895,12 @@ class Engine : public EngineBase {
       }
       PMGB_RET(fft_cols_tma<T>(n, B_, dir, zaxis ? 1 : 0, maps, bufs, nb, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));
       PMGB_CK(cudaGetLastError());
-      ColBufs<T> sb{};
-      for (int q = 0; q < nb; ++q) sb.p[q] = bufs[q] + spec_main_len(n);
-      const SeqMap ms = zaxis ? zside(n) : yside(n);
-      SeqMap none = ms;
-      none.nseq = 0;
-      PMGB_RET(fft_cols<T>(n, dir, ms, none, sb, nb, tw_, st_));
-      PMGB_CK(cudaGetLastError());
-      return PM_OK;
+      mm.nseq = 0;   // the side planes are left
     }
-    ColBufs<T> m{}, s{};
-    for (int q = 0; q < nb; ++q) {
-      m.p[q] = bufs[q];
-      s.p[q] = bufs[q] + spec_main_len(n);
-    }
-    const SeqMap mm = zaxis ? zmap(n) : ymap(n);
-    const SeqMap ms = zaxis ? zside(n) : yside(n);
-    SeqMap none = ms;
-    none.nseq = 0;
-    PMGB_RET(fft_cols<T>(n, dir, mm, none, m, nb, tw_, st_));
-    PMGB_RET(fft_cols<T>(n, dir, ms, none, s, nb, tw_, st_));
+    // one launch over the main columns (unless staged above) and the side planes
+    ColBufs<T> b{};
+    for (int q = 0; q < nb; ++q) b.p[q] = bufs[q];
+    PMGB_RET(fft_cols<T>(n, dir, mm, ms, b, nb, tw_, st_));
     PMGB_CK(cudaGetLastError());
     return PM_OK;
   }
@@ -1269,7 +1255,7 @@ class Engine : public EngineBase {
     // y forward: delta (and P_0) in place; the adjoint's P_1 and P_2 merge into
     // V = i (k_1 P_1 + k_2 P_2) in spec_[5]
     C* fwdb[2] = {spec_[0], spec_[4]};
-    prof_.begin(st_, P_COLS, pi ? 4 : 2);
+    prof_.begin(st_, P_COLS, (use_tma_ ? 2 : 1) * (pi ? 2 : 1));
     PMGB_RET(cols(nm_, -1, false, fwdb, pi ? 2 : 1));
     if (pi) PMGB_RET(cols_yx(false, spec_[5], spec_[6]));
     prof_.end(st_, P_COLS);
@@ -1285,9 +1271,9 @@ class Engine : public EngineBase {
     if (use_tma_) {
       const CUtensorMap fo[2] = {tmz_[1], tmz_[2]};   // z force, U
       PMGB_RET(fft_fused_tma<T>(nm_, false, &tmz_[0], fo, zf, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));
-      PMGB_RET(fft_fused_side<T>(nm_, zf, false, tw_, st_));
+      PMGB_RET(fft_fused_z<T>(nm_, zf, false, false, tw_, st_));
     } else {
-      PMGB_RET(fft_fused_z<T>(nm_, zf, false, tw_, st_));
+      PMGB_RET(fft_fused_z<T>(nm_, zf, false, true, tw_, st_));
     }
     prof_.end(st_, P_Z_FORCE);
     PMGB_CK(cudaGetLastError());
@@ -1302,9 +1288,9 @@ class Engine : public EngineBase {
       if (use_tma_) {
         const CUtensorMap pm2[2] = {tmz_[4], tmz_[5]};
         PMGB_RET(fft_fused_tma<T>(nm_, true, pm2, &tmz_[0], za, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));   // psi -> spec_[0]
-        PMGB_RET(fft_fused_side<T>(nm_, za, true, tw_, st_));
+        PMGB_RET(fft_fused_z<T>(nm_, za, true, false, tw_, st_));
       } else {
-        PMGB_RET(fft_fused_z<T>(nm_, za, true, tw_, st_));
+        PMGB_RET(fft_fused_z<T>(nm_, za, true, true, tw_, st_));
       }
       prof_.end(st_, P_Z_ADJ);
       PMGB_CK(cudaGetLastError());
@@ -1312,7 +1298,7 @@ class Engine : public EngineBase {
     // y inverse: z force (and psi) in place; U splits into the y force (spec_[2]) and the
     // x force before its -i k_x (spec_[3])
     C* invb[2] = {spec_[1], spec_[0]};
-    prof_.begin(st_, P_COLS, 4);
+    prof_.begin(st_, P_COLS, use_tma_ ? 4 : 2);
     PMGB_RET(cols(nm_, +1, false, invb, pi ? 2 : 1));
     PMGB_RET(cols_yx(true, spec_[2], spec_[3]));
     prof_.end(st_, P_COLS);
@@ -1333,32 +1319,22 @@ class Engine : public EngineBase {
   // u = IFFT(-i k_1 u), b = IFFT(u); merge (forward) u = i (k_1 FFT(u) + k_2 FFT(b))
   int cols_yx(bool split, C* u, C* b) {
     const int n = nm_;
-    SeqMap none = yside(n);
-    none.nseq = 0;
+    SeqMap mm = ymap(n);
     if (use_tma_) {
       const int iu = spec_index(u), ib = spec_index(b);
       if (iu < 0 || ib < 0) return PM_ERR_STATE;
-      if (split) {
-        const CUtensorMap um[2] = {tmy_[iu], tmy_[ib]};
+      const CUtensorMap um[2] = {tmy_[iu], tmy_[ib]};
+      if (split)
         PMGB_RET(fft_ysplit_tma<T>(n, B_, um, u, b, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));
-      } else {
-        const CUtensorMap pm2[2] = {tmy_[iu], tmy_[ib]};
-        PMGB_RET(fft_ymerge_tma<T>(n, B_, pm2, u, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));
-      }
-    } else if (split) {
-      PMGB_RET(fft_cols_split<T>(n, ymap(n), none, u, b, tw_, st_));
-    } else {
-      PMGB_RET(fft_cols_merge<T>(n, ymap(n), none, u, b, tw_, st_));
+      else
+        PMGB_RET(fft_ymerge_tma<T>(n, B_, um, u, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));
+      PMGB_CK(cudaGetLastError());
+      mm.nseq = 0;
     }
-    PMGB_CK(cudaGetLastError());
-    // side planes (kx = n/2): launched as side sequences, so that k_2 = 0 there
-    C* us = u + spec_main_len(n);
-    C* bs = b + spec_main_len(n);
-    if (split) {
-      PMGB_RET(fft_cols_split<T>(n, none, yside(n), us, bs, tw_, st_));
-    } else {
-      PMGB_RET(fft_cols_merge<T>(n, none, yside(n), us, bs, tw_, st_));
-    }
+    // the main columns (unless staged above) and the side planes (kx = n/2: side
+    // sequences, so that k_2 = 0 there) in one launch
+    PMGB_RET(split ? fft_cols_split<T>(n, mm, yside(n), u, b, tw_, st_)
+                   : fft_cols_merge<T>(n, mm, yside(n), u, b, tw_, st_));
     PMGB_CK(cudaGetLastError());
     return PM_OK;
   }
@@ -1386,7 +1362,7 @@ class Engine : public EngineBase {
   // 2LPT (Sec. 2.1, Eqs. 2-4) from Omega^ in spec_[0]: the Hessian of the first-order
   // potential in two groups of three (diagonal, mixed) through spec_[1..3], the source S
   // accumulated in the real view of spec_[4], s2_c = IDFT[i k_c / k^2 S^] / n^3 through
-  // spec_[1..3], then s += D2 s2, p += G_D2 s2.  26 launches.
+  // spec_[1..3], then s += D2 s2, p += G_D2 s2.  18 launches.
   int lpt2_state() {
     const long long lis = spec_len_cx(np_);
     C* h[3] = {spec_[1], spec_[2], spec_[3]};
@@ -1413,7 +1389,7 @@ class Engine : public EngineBase {
   // and the partials xi_0.s2, pi_0.s2; S_bar = sum_c IDFT[conj(i k_c / k^2) DFT sbar2_c] / n^3
   // (real view of spec_[4]); per Hessian group phi_bar = dS/dphi S_bar, and
   // sum_ij k_i k_j / k^2 amp DFT phi_bar_ij accumulated in spec_[5], where the Zel'dovich
-  // transpose adds its part.  Leaves Omega^ in spec_[0].  39 launches.
+  // transpose adds its part.  Leaves Omega^ in spec_[0].  27 launches.
   int lpt2_adjoint() {
     const long long lis = spec_len_cx(np_);
     k_ic_adj_prep<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(xi_, pi_, s2_, N_, d2_, gd2_, rmesh(1), rmesh(2),

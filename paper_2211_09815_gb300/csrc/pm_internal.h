@@ -10,7 +10,7 @@
 namespace pmgb {
 
 // Address map of a batch of length-L sequences for a column FFT pass.  Sequence s,
-// element r lives at  o1*os1 + o0*os0 + col*cs + r*es  (complex elements) with
+// element r lives at  off + o1*os1 + o0*os0 + col*cs + r*es  (complex elements) with
 // col = s % ncols, o0 = (s / ncols) % n0, o1 = s / (ncols * n0).
 struct SeqMap {
   long long es, cs;
@@ -19,6 +19,7 @@ struct SeqMap {
   int n0;
   long long os1;
   int nseq;
+  long long off;
 };
 
 template <typename T> struct ColBufs { cx_t<T>* p[4]; };
@@ -67,8 +68,9 @@ int fft_x_c2r(int n, const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* t
 template <typename T>
 int fft_x_c2r4(int n, const RowJob<T>& job, int nrows, int dq, void* out, signed char* fexp, const cx_t<T>* tw,
                cudaStream_t st);
+// (main = false: the side-plane (kx = n/2) columns only, beside a TMA-staged pass)
 template <typename T>
-int fft_fused_z(int n, const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st);
+int fft_fused_z(int n, const ZJob<T>& job, bool adjoint, bool main, const cx_t<T>* tw, cudaStream_t st);
 
 // Bounded mbarrier waits of the TMA-staged passes: the device flag a wait that gives up
 // sets, and the spin limit of each CTA's first wait (negative: the normal limit; a test
@@ -94,9 +96,6 @@ int fft_ysplit_tma(int n, int batch, const CUtensorMap* umaps, cx_t<T>* u, cx_t<
 template <typename T>
 int fft_ymerge_tma(int n, int batch, const CUtensorMap* pmaps, cx_t<T>* p1, const cx_t<T>* tw, const WaitCtl& wc, int nsm,
                    cudaStream_t st);
-// the side-plane (kx = n/2) tiles of the fused z passes only
-template <typename T>
-int fft_fused_side(int n, const ZJob<T>& job, bool adjoint, const cx_t<T>* tw, cudaStream_t st);
 // tensor maps of one spectrum buffer for the y pass (box along y) and the z pass (box along z)
 template <typename T>
 int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap);
