@@ -1154,7 +1154,7 @@ class Engine : public EngineBase {
               const SepTargets* tg = nullptr) {
     if (pi) {
       prof_.begin(st_, P_OTHER, 1);
-      k_pi_exponents<<<1, 64, 0, st_>>>(pimax_, e_pi_, 3 * B_, fixed_top<T>(lgN_));
+      k_pi_exponents<<<(3 * B_ + 63) / 64, 64, 0, st_>>>(pimax_, e_pi_, 3 * B_, fixed_top<T>(lgN_));
       prof_.end(st_, P_OTHER);
       PMGB_CK(cudaGetLastError());
       PMGB_CK(cudaMemsetAsync(pimax_, 0, sizeof(unsigned) * 3 * B_, st_));
