@@ -206,15 +206,6 @@ constexpr int kRangeCv[20] = {0, 1, 3, 5, 7, 2, 3, 6, 7, 3, 7, 4, 5, 6, 7, 5, 7,
 constexpr unsigned long long kRangeD = pack3(kRangeDv);
 constexpr unsigned long long kRangeC = pack3(kRangeCv);
 
-// Exact 64-bit addition into a shared accumulator kept as two 32-bit words: the low word
-// takes a native 32-bit atomic add whose returned old value gives the carry, the high word
-// the high part plus that carry.  Each addition is exact mod 2^64, so the final pair holds
-// the exact sum in any order (64-bit shared atomics are several times slower).
-__device__ __forceinline__ void smem_add64(unsigned* lo, unsigned* hi, unsigned vl, unsigned vh) {
-  const unsigned old = atomicAdd(lo, vl);
-  const unsigned h = vh + (old + vl < old ? 1u : 0u);
-  if (h) atomicAdd(hi, h);
-}
 // the exact sum (two words) in the working precision, correctly rounded; sums that fit in
 // 32 bits take one hardware conversion
 template <typename T> __device__ __forceinline__ T words_to_real(unsigned lo, unsigned hi);

@@ -63,6 +63,16 @@ __device__ __forceinline__ long long f2ll_rn(float v) {
   return (b >> 31) ? -(long long)r : (long long)r;
 }
 
+// Exact 64-bit addition into a shared accumulator kept as two 32-bit words: the low word
+// takes a native 32-bit atomic add whose returned old value gives the carry, the high word
+// the high part plus that carry.  Each addition is exact mod 2^64, so the final pair holds
+// the exact sum in any order (64-bit shared atomics are several times slower).
+__device__ __forceinline__ void smem_add64(unsigned* lo, unsigned* hi, unsigned vl, unsigned vh) {
+  const unsigned old = atomicAdd(lo, vl);
+  const unsigned h = vh + (old + vl < old ? 1u : 0u);
+  if (h) atomicAdd(hi, h);
+}
+
 // 2^e built from its bit pattern, for e in the normal range of T (the FP64 pipe that
 // ldexp goes through is slow on this part)
 template <typename T> __device__ __forceinline__ T pow2i(int e);

@@ -522,9 +522,10 @@ class Engine : public EngineBase {
     PMGB_CK(cudaMemcpyAsync(dt, tgt, sizeof(double) * B_ * nb, cudaMemcpyDefault, st_));
     PMGB_CK(cudaMemcpyAsync(dw, w, sizeof(double) * B_ * nb, cudaMemcpyDefault, st_));
     const double vol = cfg_.box * cfg_.box * cfg_.box;
-    k_power_loss<<<(B_ + 31) / 32, 32, 0, st_>>>(pw_out_, pw_out_ + (B_ + 1) * nb, dt, dw, nb, B_,
-                                                 2.0 * vol / ((double)M_ * (double)M_), dl, dg);
-    k_power_grad<T><<<dim3(512, B_), 256, 0, st_>>>(spec_[6], nm_, spec_len_cx(nm_), nb, dg);
+    k_power_loss<<<B_, kPowerThreads, 0, st_>>>(pw_out_, pw_out_ + (B_ + 1) * nb, dt, dw, nb,
+                                                2.0 * vol / ((double)M_ * (double)M_), dl, dg);
+    const PowerRuns pr = power_runs(nm_, spec_lzb(nm_));
+    k_power_grad<T><<<dim3(power_grid(pr), B_), kPowerThreads, 0, st_>>>(spec_[6], pr, spec_len_cx(nm_), nb, dg);
     PMGB_CK(cudaGetLastError());
     PMGB_RET(c2r_real(nm_, spec_[6], (T*)djdd, M_));
     if (loss) {
@@ -538,25 +539,38 @@ class Engine : public EngineBase {
   // spec_[6].  Deterministic: per-bin int64 fixed point scaled from a first max pass.
   int power_dev(const T* d) {
     const int nb = nm_ / 2;
-    if (!pw_acc_) PMGB_RET(alloc(&pw_acc_, (long long)(B_ + 2) * nb));
+    if (!pw_acc_) PMGB_RET(alloc(&pw_acc_, (long long)B_ * nb));
     if (!pw_max_) PMGB_RET(alloc(&pw_max_, (long long)B_ * nb));
-    if (!pw_e_) PMGB_RET(alloc(&pw_e_, (long long)B_ * nb));
     if (!pw_out_) PMGB_RET(alloc(&pw_out_, (long long)(B_ + 2) * nb));
+    if (!pw_modes_) {
+      // the modes of each bin: constants of the mesh side, counted once per context
+      unsigned long long* m = nullptr;
+      PMGB_RET(alloc(&m, 2LL * nb));
+      PMGB_CK(cudaMemsetAsync(m, 0, sizeof(unsigned long long) * 2 * nb, st_));
+      k_power_modes<<<std::min(4 * nsm_, (nb * nb + kPowerThreads - 1) / kPowerThreads), kPowerThreads, 0, st_>>>(
+          nb, m, m + nb);
+      PMGB_CK(cudaGetLastError());
+      pw_modes_ = m;
+    }
     PMGB_RET(r2c_real(nm_, d, M_, spec_[6]));
-    PMGB_CK(cudaMemsetAsync(pw_acc_, 0, sizeof(unsigned long long) * (B_ + 2) * nb, st_));
+    PMGB_CK(cudaMemsetAsync(pw_acc_, 0, sizeof(unsigned long long) * B_ * nb, st_));
     PMGB_CK(cudaMemsetAsync(pw_max_, 0, sizeof(unsigned) * B_ * nb, st_));
     const long long is = spec_len_cx(nm_);
-    k_power_max<T><<<dim3(512, B_), 256, 0, st_>>>(spec_[6], nm_, is, nb, pw_max_);
-    k_power_exponents<<<(B_ * nb + 255) / 256, 256, 0, st_>>>(pw_max_, pw_e_, B_ * nb, ilog2(M_));
-    k_power_acc<T><<<dim3(512, B_), 256, 0, st_>>>(spec_[6], nm_, is, nb, pw_e_, pw_acc_, pw_acc_ + B_ * nb,
-                                                  pw_acc_ + (B_ + 1) * nb);
+    const PowerRuns pr = power_runs(nm_, spec_lzb(nm_));
+    const dim3 grid(power_grid(pr), B_);
+    k_power_max<T><<<grid, kPowerThreads, 0, st_>>>(spec_[6], pr, is, nb, pw_max_);
+    k_power_acc<T><<<grid, kPowerThreads, 0, st_>>>(spec_[6], pr, is, nb, ilog2(M_), pw_max_, pw_acc_);
     const double vol = cfg_.box * cfg_.box * cfg_.box;
-    k_power_final<<<(B_ * nb + 255) / 256, 256, 0, st_>>>(pw_acc_, pw_acc_ + B_ * nb, pw_acc_ + (B_ + 1) * nb, pw_e_,
-                                                        nb, B_, vol / ((double)M_ * (double)M_),
-                                                        2.0 * M_PI / cfg_.box, pw_out_, pw_out_ + B_ * nb,
-                                                        pw_out_ + (B_ + 1) * nb);
+    k_power_final<T><<<(B_ * nb + 255) / 256, 256, 0, st_>>>(pw_acc_, pw_modes_, pw_modes_ + nb, pw_max_, ilog2(M_),
+                                                           nb, B_, vol / ((double)M_ * (double)M_),
+                                                           2.0 * M_PI / cfg_.box, pw_out_, pw_out_ + B_ * nb,
+                                                           pw_out_ + (B_ + 1) * nb);
     PMGB_CK(cudaGetLastError());
     return PM_OK;
+  }
+  // four resident blocks per SM: each block adds its bins to the global ones once
+  int power_grid(const PowerRuns& pr) const {
+    return (int)std::min<long long>(4LL * nsm_, (pr.count + kPowerThreads - 1) / kPowerThreads);
   }
 
   // One gradient evaluation on device buffers, captured once into a CUDA graph on the
@@ -1510,7 +1524,7 @@ class Engine : public EngineBase {
   T *tgt_ = nullptr, *djdd_ = nullptr, *gw_ = nullptr;
   unsigned long long* pw_acc_ = nullptr;
   unsigned* pw_max_ = nullptr;
-  int* pw_e_ = nullptr;
+  unsigned long long* pw_modes_ = nullptr;   // modes and sum of |n| of each power bin
   double* pw_out_ = nullptr;
   double* pl_buf_ = nullptr;   // power objective: target, weights, g, loss
   std::vector<int> snap_of_;   // observed states: step -> snapshot index (-1: none)
