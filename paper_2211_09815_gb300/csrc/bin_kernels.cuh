@@ -206,13 +206,48 @@ constexpr int kRangeCv[20] = {0, 1, 3, 5, 7, 2, 3, 6, 7, 3, 7, 4, 5, 6, 7, 5, 7,
 constexpr unsigned long long kRangeD = pack3(kRangeDv);
 constexpr unsigned long long kRangeC = pack3(kRangeCv);
 
-// the exact sum (two words) in the working precision, correctly rounded; sums that fit in
-// 32 bits take one hardware conversion
+// Contributions of the NQ quantities of one CIC corner, added exactly to the tile's
+// accumulators (word pairs at loc, loc + cells, ... of lo and hi).
+//
+// FP32 contributions are int32 (fixed_top), and a pair holds the sum hi 2^32 + lo with lo
+// SIGNED: hi changes only when lo overflows, about once per 4 units of weight, and for pi
+// sums, whose terms have both signs, hardly ever.  (With an unsigned low word every negative
+// term borrowed from the high one: half of the pi atomics were high-word ones.)  The
+// corner's atomics are all issued before the first returned value is looked at.
+// FP64 contributions carry their own high word.
+template <int NQ> __device__ __forceinline__ void corner_add(unsigned* lo, unsigned* hi, int cells, int loc,
+                                                             const float (&x)[NQ]) {
+  int v[NQ], old[NQ], over = 0;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) v[q] = __float2int_rn(x[q]);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) old[q] = atomicAdd(reinterpret_cast<int*>(lo) + q * cells + loc, v[q]);
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int s = (int)((unsigned)old[q] + (unsigned)v[q]);
+    v[q] = (old[q] ^ s) & (v[q] ^ s);   // negative: the signed sum overflowed
+    over |= v[q];
+  }
+  if (over < 0) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (v[q] < 0) atomicAdd(hi + q * cells + loc, old[q] < 0 ? 0xFFFFFFFFu : 1u);
+  }
+}
+template <int NQ> __device__ __forceinline__ void corner_add(unsigned* lo, unsigned* hi, int cells, int loc,
+                                                             const double (&x)[NQ]) {
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const unsigned long long r = (unsigned long long)__double2ll_rn(x[q]);
+    smem_add64(lo + q * cells + loc, hi + q * cells + loc, (unsigned)r, (unsigned)(r >> 32));
+  }
+}
+// the exact sum (two words, as accumulated above) in the working precision, correctly
+// rounded; FP32 sums that fit in 32 bits take one hardware conversion
 template <typename T> __device__ __forceinline__ T words_to_real(unsigned lo, unsigned hi);
 template <> __device__ __forceinline__ float words_to_real<float>(unsigned lo, unsigned hi) {
-  if (hi == 0u) return __uint2float_rn(lo);
-  if (hi == 0xFFFFFFFFu && (lo >> 31)) return __int2float_rn((int)lo);
-  return ll2f_rn((long long)(((unsigned long long)hi << 32) | lo));
+  if (hi == 0u) return __int2float_rn((int)lo);
+  return ll2f_rn((long long)((unsigned long long)hi << 32) + (int)lo);
 }
 template <> __device__ __forceinline__ double words_to_real<double>(unsigned lo, unsigned hi) {
   return (double)(long long)(((unsigned long long)hi << 32) | lo);
@@ -259,17 +294,13 @@ __device__ __forceinline__ void pull_accumulate(const BinGeo& bg, const V4<T>* _
   const T sd = pow2i<T>(e_d);
   const unsigned total = rpre[20];
   const unsigned mx = (1u << bg.lx) - 1, my = (1u << bg.ly) - 1, mz = (1u << bg.lz) - 1;
+  int r = 0;   // range of f (f only grows)
   for (unsigned f = threadIdx.x; f < total; f += blockDim.x) {
-    int r = 0;
     while (f >= rpre[r + 1]) ++r;
     const unsigned d = (unsigned)((kRangeD >> (3 * r)) & 7u);
     const unsigned pos = rbeg[r] + (f - rpre[r]);
     const V4<T> r0 = rec0[pos];
-    const T t[3] = {r0.x, r0.y, r0.z};
     const unsigned packed = real_to_bits<T>(r0.w);
-    const int l0 = (int)(packed >> 20), l1 = (int)((packed >> 10) & 1023u), l2 = (int)(packed & 1023u);
-    const unsigned cls = (unsigned)((unsigned)l2 == mx) | ((unsigned)((unsigned)l1 == my) << 1) |
-                         ((unsigned)((unsigned)l0 == mz) << 2);
     T pv[3] = {0, 0, 0};
     if constexpr (NQ == 4) {
       const V4<T> r1 = rec1[pos];
@@ -277,28 +308,28 @@ __device__ __forceinline__ void pull_accumulate(const BinGeo& bg, const V4<T>* _
       pv[1] = r1.y;
       pv[2] = r1.z;
     }
+    // Per axis: a particle of this tile (bit of d clear) has its lower corner at its own
+    // cell l and, unless that is the tile's last layer, the upper one at l + 1; one of the
+    // lower neighbour (bit set) has its upper corner on the tile's first layer.
+    const int l0 = (int)(packed >> 20), l1 = (int)((packed >> 10) & 1023u), l2 = (int)(packed & 1023u);
+    const bool up0 = !(d & 4u) && (unsigned)l0 != mz, up1 = !(d & 2u) && (unsigned)l1 != my,
+               up2 = !(d & 1u) && (unsigned)l2 != mx;
+    const T wa[2] = {(d & 4u) ? r0.x : (T)1 - r0.x, r0.x}, wb[2] = {(d & 2u) ? r0.y : (T)1 - r0.y, r0.y},
+            wc[2] = {(d & 1u) ? r0.z : (T)1 - r0.z, r0.z};
+    const int base = ((((d & 4u) ? 0 : l0) << bg.ly) + ((d & 2u) ? 0 : l1)) << bg.lx;
+    const int loc0 = base + ((d & 1u) ? 0 : l2);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      // corner e (bit 2: axis 0, bit 1: axis 1, bit 0: axis 2) crosses into the next tile
-      // along an axis iff the cell is on the tile's last layer there and the corner is the
-      // upper one; it lands in this CTA's tile iff those crossings equal d
-      const unsigned carry = cls & (unsigned)e;
-      if (carry != d) continue;
-      const int a0 = (d & 4u) ? 0 : l0 + ((e >> 2) & 1);
-      const int a1 = (d & 2u) ? 0 : l1 + ((e >> 1) & 1);
-      const int a2 = (d & 1u) ? 0 : l2 + (e & 1);
-      const int loc = (((a0 << bg.ly) + a1) << bg.lx) + a2;
-      const T w = ((e & 4) ? t[0] : (T)1 - t[0]) * ((e & 2) ? t[1] : (T)1 - t[1]) * ((e & 1) ? t[2] : (T)1 - t[2]);
-      unsigned vl, vh;
-      fixed_words<T>(w * sd, vl, vh);
-      smem_add64(acc + loc, hacc + loc, vl, vh);
+      if (((e & 4) && !up0) || ((e & 2) && !up1) || ((e & 1) && !up2)) continue;
+      const int loc = loc0 + ((e & 4) ? 1 << (bg.lx + bg.ly) : 0) + ((e & 2) ? 1 << bg.lx : 0) + (e & 1);
+      const T w = wa[e >> 2] * wb[(e >> 1) & 1] * wc[e & 1];
+      T x[NQ];
+      x[0] = w * sd;
       if constexpr (NQ == 4) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          fixed_words<T>(pv[c] * w, vl, vh);
-          smem_add64(acc + (1 + c) * cells + loc, hacc + (1 + c) * cells + loc, vl, vh);
-        }
+        for (int c = 0; c < 3; ++c) x[1 + c] = pv[c] * w;
       }
+      corner_add<NQ>(acc, hacc, cells, loc, x);
     }
   }
   __syncthreads();

@@ -266,22 +266,6 @@ template <typename T> inline int fixed_top(int lgN);
 template <> inline int fixed_top<float>(int lgN) { return 61 - lgN < 30 ? 61 - lgN : 30; }
 template <> inline int fixed_top<double>(int lgN) { return 61 - lgN; }
 
-// A fixed-point contribution as the two 32-bit words of an int64, correctly rounded
-// (nearest-even).  FP32 contributions are at most 2^30 in magnitude (fixed_top), so one
-// hardware conversion to int32 rounds them (ties to even, symmetric in the sign) and the
-// high word is the sign extension.
-template <typename T> __device__ __forceinline__ void fixed_words(T v, unsigned& lo, unsigned& hi);
-template <> __device__ __forceinline__ void fixed_words<float>(float v, unsigned& lo, unsigned& hi) {
-  const int r = __float2int_rn(v);
-  lo = (unsigned)r;
-  hi = (unsigned)(r >> 31);
-}
-template <> __device__ __forceinline__ void fixed_words<double>(double v, unsigned& lo, unsigned& hi) {
-  const unsigned long long r = (unsigned long long)__double2ll_rn(v);
-  lo = (unsigned)r;
-  hi = (unsigned)(r >> 32);
-}
-
 // ------------------------------------------------------------------ deposit bins
 // Bins of the tile-owner deposit (bin_kernels.cuh): mesh tiles of 2^lx x 2^ly x 2^lz cells
 // (x = array axis 2), and per tile a class of three bits, set when the particle's cell is on
