@@ -12,6 +12,7 @@
 #include <cuda_fp16.h>
 
 #include "fft.cuh"
+#include "fft_rows.cuh"
 #include "fft_tma.cuh"
 #include "pm_internal.h"
 
@@ -658,7 +659,9 @@ static void launch_r2c_S(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T
 }
 template <typename T, int L>
 static void launch_r2c_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
-  if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
+  if constexpr (sizeof(T) == 4 && has_warp_rows_r2c(L))
+    launch_rows_r2c<L>(job, nbuf, nrows, tw, st);
+  else if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
     launch_r2c_S<T, L, true>(job, nbuf, nrows, tw, st);
   else
     launch_r2c_S<T, L, false>(job, nbuf, nrows, tw, st);
@@ -675,7 +678,9 @@ static void launch_c2r_S(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T
 }
 template <typename T, int L>
 static void launch_c2r_L(const RowJob<T>& job, int nbuf, int nrows, const cx_t<T>* tw, cudaStream_t st) {
-  if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
+  if constexpr (sizeof(T) == 4 && has_warp_rows(L))
+    launch_rows_c2r<L>(job, nbuf, nrows, tw, st);
+  else if (small_tiles((long long)nbuf * tiles_for(nrows, RowTile<T, L>::TR)))
     launch_c2r_S<T, L, true>(job, nbuf, nrows, tw, st);
   else
     launch_c2r_S<T, L, false>(job, nbuf, nrows, tw, st);
@@ -915,7 +920,9 @@ static void launch_c2r4_LQ(const RowJob<T>& job, int nrows, int dq, void* out, s
                            cudaStream_t st) {
   using TL = C2R4Tile<T, L, Q>;
   if constexpr (RowTile<T, L>::TR % 4 == 0 && (TL::TR * L) % TL::P::RMAX == 0) {
-    if (small_tiles(tiles_for(nrows, TL::RT)))
+    // (its tiles hold Q rows of work each: small ones only below one full tile per SM; FP64
+    // at 64^3, 256 tiles: 23 us full, 27 us small)
+    if (tiles_for(nrows, TL::RT) < kNumSms)
       launch_c2r4_S<T, L, Q, true>(job, nrows, dq, out, fexp, tw, st);
     else
       launch_c2r4_S<T, L, Q, false>(job, nrows, dq, out, fexp, tw, st);
@@ -924,6 +931,11 @@ static void launch_c2r4_LQ(const RowJob<T>& job, int nrows, int dq, void* out, s
 template <typename T, int L>
 static void launch_c2r4_L(const RowJob<T>& job, int nrows, int dq, void* out, signed char* fexp, const cx_t<T>* tw,
                           cudaStream_t st) {
+  if constexpr (sizeof(T) == 4 && has_warp_rows(L)) {
+    if (!job.b[3].spec) return launch_rows_c2r4<L, 3>(job, nrows, dq, out, fexp, tw, st);
+    // (four components of 128 points: 16 x 256^3 in 1.64 ms as tiles, 1.68 as rows)
+    if constexpr (L != 128) return launch_rows_c2r4<L, 4>(job, nrows, dq, out, fexp, tw, st);
+  }
   if (job.b[3].spec) launch_c2r4_LQ<T, L, 4>(job, nrows, dq, out, fexp, tw, st);
   else launch_c2r4_LQ<T, L, 3>(job, nrows, dq, out, fexp, tw, st);
 }

@@ -11,7 +11,10 @@
 //
 // What bounds these passes is HBM; the tile form they replace (fft_impl.cuh, still used for
 // FP64 and for shorter rows) moved each row through shared memory three times, with two of
-// five wavefronts lost to bank conflicts in the three-component C2R.
+// five wavefronts lost to bank conflicts in the three-component C2R.  The R2C takes this form
+// at L = 512 only (four buffers of 1024^3: 7.5 -> 5.3 ms, where the tile form has two 64 KB
+// tiles per SM); below, the tile form splits and stores with fewer instructions (512^3, four
+// buffers: 750 us, this form 867).
 #pragma once
 #include <cuda_fp16.h>
 
@@ -28,6 +31,7 @@ template <> struct WarpRow<256> { static constexpr int LANES = 16, R0 = 16, R1 =
 template <> struct WarpRow<512> { static constexpr int LANES = 32, R0 = 8,  R1 = 8,  R2 = 8, BUF = 576; };
 
 constexpr bool has_warp_rows(int L) { return L >= 64 && L <= 512; }
+constexpr bool has_warp_rows_r2c(int L) { return L == 512; }
 
 template <int L> struct RowShape : WarpRow<L> {
   using W = WarpRow<L>;
@@ -55,9 +59,23 @@ __device__ __forceinline__ void row_tables(float2* t, float2* wn, const float2* 
   __syncthreads();
 }
 
-template <int DIR> __device__ __forceinline__ float2 tw_dir(float2 w) {
-  if (DIR > 0) w.y = -w.y;
-  return w;
+// Products with their roundings written out (which of the two terms is rounded on its own), so
+// that they do not depend on what the compiler contracts around them: the row forms round like
+// the tile forms.
+__device__ __forceinline__ float2 cmul_fwd(float2 a, float2 b) {
+  return cmake<float2>(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float2 cmul_inv(float2 a, float2 b) {
+  return cmake<float2>(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ float2 cadd_rn(float2 a, float2 b) {
+  return cmake<float2>(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+
+// v exp(DIR 2 pi i m / L) from the table's exp(-2 pi i m / L)
+template <int DIR> __device__ __forceinline__ float2 tw_mul(float2 v, float2 w) {
+  if constexpr (DIR > 0) return cmul_inv(v, cconj(w));
+  return cmul_fwd(v, w);
 }
 
 // Length-L DFT of the row held as z[r] = element j + LANES r, in and out, through the row's
@@ -88,7 +106,7 @@ __device__ __forceinline__ void row_fft(float2 (&z)[RowShape<L>::P], float2* buf
 #pragma unroll
       for (int r = 0; r < 8; ++r) v[s][r] = buf[i + (i >> 4) + 68 * r];
 #pragma unroll
-      for (int r = 1; r < 8; ++r) v[s][r] = cmul(v[s][r], tw_dir<DIR>(t[L + 8 * r + (j & 7)]));
+      for (int r = 1; r < 8; ++r) v[s][r] = tw_mul<DIR>(v[s][r], t[L + 8 * r + (j & 7)]);
       dft<8, DIR>(v[s]);
     }
     __syncwarp();
@@ -105,7 +123,7 @@ __device__ __forceinline__ void row_fft(float2 (&z)[RowShape<L>::P], float2* buf
 #pragma unroll
       for (int r = 0; r < 8; ++r) v[s][r] = buf[i + 72 * r];
 #pragma unroll
-      for (int r = 1; r < 8; ++r) v[s][r] = cmul(v[s][r], tw_dir<DIR>(t[64 * r + i]));
+      for (int r = 1; r < 8; ++r) v[s][r] = tw_mul<DIR>(v[s][r], t[64 * r + i]);
       dft<8, DIR>(v[s]);
 #pragma unroll
       for (int r = 0; r < 8; ++r) z[2 * r + s] = v[s][r];
@@ -125,7 +143,7 @@ __device__ __forceinline__ void row_fft(float2 (&z)[RowShape<L>::P], float2* buf
 #pragma unroll
       for (int r = 0; r < R1; ++r) v[r] = buf[i + (R0 + 1) * r];
 #pragma unroll
-      for (int r = 1; r < R1; ++r) v[r] = cmul(v[r], tw_dir<DIR>(t[R0 * r + i]));
+      for (int r = 1; r < R1; ++r) v[r] = tw_mul<DIR>(v[r], t[R0 * r + i]);
       dft<R1, DIR>(v);
 #pragma unroll
       for (int r = 0; r < R1; ++r) z[K * r + s] = v[r];
@@ -183,17 +201,23 @@ k_rows_r2c(RowJob<float> job, int nrows, int nbuf, const float2* __restrict__ tw
 #pragma unroll
     for (int r = 0; r < P; ++r) z[r] = in[j + LN * r];
     row_fft<L, -1>(z, buf, j, t);
-    // even/odd split: X[k] = E + W^k O, E = (Z[k] + conj Z[L-k]) / 2, O = -i (Z[k] - conj Z[L-k]) / 2
+    // even/odd split of the pairs k, L - k with k < L/2: X[k] = E + W^k O, X[L-k] = conj(E - W^k O),
+    // E = (Z[k] + conj Z[L-k]) / 2, O = -i (Z[k] - conj Z[L-k]) / 2; lane 0 has the middle k = L/2
+    // (its own partner) besides
 #pragma unroll
-    for (int r = 0; r < P; ++r) {
+    for (int r = 0; r <= P / 2; ++r) {
+      if (r == P / 2 && j != 0) break;
       const int k = j + LN * r;
-      const float2 zk = z[r], zm = row_partner<L>(z, r, j, z[0]);
+      const float2 zk = z[r], zm = r < P / 2 ? row_partner<L>(z, r, j, z[0]) : zk;
       const float2 e = cscale(cadd(zk, cconj(zm)), 0.5f);
       const float2 d = cscale(csub(zk, cconj(zm)), 0.5f);
-      float2 x = cadd(e, cmul(wn[k], cmake<float2>(d.y, -d.x)));
+      const float2 wo = cmul_fwd(wn[k], cmake<float2>(d.y, -d.x));
+      float2 x = cadd_rn(e, wo);
       if (r == 0 && j == 0) {
         x = cmake<float2>(zk.x + zk.y, 0.f);
         rb.spec[pl.side] = cmake<float2>(zk.x - zk.y, 0.f);
+      } else if (r < P / 2) {
+        out[L - k] = cmake<float2>(__fsub_rn(e.x, wo.x), -__fsub_rn(e.y, wo.y));
       }
       out[k] = x;
     }
@@ -221,8 +245,8 @@ __device__ __forceinline__ void row_untangle(float2 (&x)[RowShape<L>::P], float2
     const int k = j + LN * r;
     const float2 xk = x[r], xm = row_partner<L>(x, r, j, xl);
     const float2 e = cadd(xk, cconj(xm));
-    const float2 o = cmul(csub(xk, cconj(xm)), cconj(wn[k]));
-    z[r] = cadd(e, cmul_i(o));
+    const float2 o = cmul_inv(csub(xk, cconj(xm)), cconj(wn[k]));
+    z[r] = cadd_rn(e, cmul_i(o));
     if (r == 0 && j == 0) z[r] = cmake<float2>(xk.x + xm.x, xk.x - xm.x);
   }
 #pragma unroll
@@ -259,6 +283,18 @@ k_rows_c2r(RowJob<float> job, int nrows, int nbuf, const float2* __restrict__ tw
   }
 }
 
+// asynchronous copies into shared memory (the calling thread's groups)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int K> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory"); }
+
 // 32-byte store (both cells of one complex value of the row)
 __device__ __forceinline__ void store_cells(V4<float>* p, V4<float> a, V4<float> b) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
@@ -268,36 +304,90 @@ __device__ __forceinline__ void store_cells(V4<float>* p, V4<float> a, V4<float>
 
 // C2R of Q = 3 or 4 components of a row, written as one V4 per cell ([cell](c0, c1, c2, c3),
 // c3 = 0 for Q = 3) straight from the registers that hold them all: component after component
-// runs through the row's buffer, then every lane stores whole 32-byte pairs of cells.
+// runs through a buffer of its own, then every lane stores whole 32-byte pairs of cells.
 // Component dq (none if dq < 0) is multiplied by -i k_x on the way in.
+//
+// Q = 4 leaves registers for two blocks of 128 threads per SM, too few warps to hide the loads
+// behind the transforms, so its loads are asynchronous copies: once a component's buffer has
+// served its exchange, the same component of the warp's next row is copied into it, a whole row
+// ahead of its use.  Q = 3 (three blocks) reads plainly, all through one buffer.
+// Measured at 512^3, tile form -> this: Q = 3 753 -> 569 us (590 with asynchronous copies), Q = 4
+// 829 -> 703 us (851 with plain loads), against 550 and 640 us for their bytes at the copy
+// bandwidth.
+//
 // H: the FP16 force mesh (pm_config.half_force): per cell four halves, each field of a row
 // scaled by 2^-e so that the row's largest magnitude lies in [2^14, 2^15), e stored as one int8
 // per (row, field) in fexp ([rows][4]).
+template <int Q> constexpr int kRows4Bufs = Q == 4 ? Q : 1;   // buffers per row
+template <int L, int Q> constexpr int kRows4Smem = (RowShape<L>::RPB * kRows4Bufs<Q> * RowShape<L>::BUF + RowShape<L>::TW + L) *
+                                                   (int)sizeof(float2);
 template <int L, int Q, bool H>
 __global__ void __launch_bounds__(RowShape<L>::NT, Q == 4 ? 2 : 3)
 k_rows_c2r4(RowJob<float> job, int nrows, int dq, void* __restrict__ out, signed char* __restrict__ fexp,
             const float2* __restrict__ twL, const float2* __restrict__ twN) {
   using S = RowShape<L>;
   constexpr int N = 2 * L, P = S::P, LN = S::LANES;
+  constexpr int NB = kRows4Bufs<Q>;
+  constexpr bool ASYNC = NB > 1;
+  static_assert(S::BUF > L, "room for the side element");
   extern __shared__ __align__(16) float2 rsm[];
-  float2* t = rsm + S::RPB * S::BUF;
+  float2* t = rsm + S::RPB * NB * S::BUF;
   float2* wn = t + S::TW;
-  row_tables<L>(t, wn, twL, twN);
   const int lane = threadIdx.x & 31, j = lane & (LN - 1);
   const int lrow = threadIdx.x / LN;
-  float2* buf = rsm + lrow * S::BUF;
+  float2* bufs = rsm + lrow * NB * S::BUF;
   const int groups = nrows / S::RPB;
+  // component q of the row whose main and side offsets are given (main < 0: none), as one group
+  auto fetch = [&](int q, long long main, long long side) {
+    if (main >= 0) {
+      float2* b = bufs + q * S::BUF;
+      const float2* in = job.b[q].spec + main;
+#pragma unroll
+      for (int r = 0; r < P / 2; ++r) cp_async16(b + 2 * (j + LN * r), in + 2 * (j + LN * r));
+      if (j == 0) cp_async8(b + L, job.b[q].spec + side);
+    }
+    cp_async_commit();
+  };
+  auto place = [&](int g, long long& main, long long& side) {
+    if (g < groups) {
+      const RowPlace<L> pl(g * S::RPB + lrow, job.lzb);
+      main = pl.main, side = pl.side;
+    } else {
+      main = side = -1;
+    }
+  };
+  long long nmain, nside;
+  place(blockIdx.x, nmain, nside);
+  if constexpr (ASYNC) {
+#pragma unroll
+    for (int q = 0; q < Q; ++q) fetch(q, nmain, nside);
+  }
+  row_tables<L>(t, wn, twL, twN);
   for (int g = blockIdx.x; g < groups; g += gridDim.x) {
     const int row = g * S::RPB + lrow;
-    const RowPlace<L> pl(row, job.lzb);
+    const long long main = nmain, side = nside;
+    place(g + gridDim.x, nmain, nside);
     float2 f[Q][P];
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
-      const float2* in = job.b[q].spec + pl.main;
+      float2* b = bufs + (ASYNC ? q : 0) * S::BUF;
+      float2 xl;
+      if constexpr (ASYNC) {
+        cp_async_wait<Q - 1>();      // this component's copies; the Q - 1 groups behind it may be in flight
+        __syncwarp();
 #pragma unroll
-      for (int r = 0; r < P; ++r) f[q][r] = in[j + LN * r];
-      row_untangle<L>(f[q], job.b[q].spec[pl.side], j, q == dq, wn);
-      row_fft<L, +1>(f[q], buf, j, t);
+        for (int r = 0; r < P; ++r) f[q][r] = b[j + LN * r];
+        xl = b[L];
+        __syncwarp();                // read by every lane before the exchange overwrites it
+      } else {
+        const float2* in = job.b[q].spec + main;
+#pragma unroll
+        for (int r = 0; r < P; ++r) f[q][r] = in[j + LN * r];
+        xl = job.b[q].spec[side];
+      }
+      row_untangle<L>(f[q], xl, j, q == dq, wn);
+      row_fft<L, +1>(f[q], b, j, t);
+      if constexpr (ASYNC) fetch(q, nmain, nside);
     }
     if constexpr (!H) {
       V4<float>* o = reinterpret_cast<V4<float>*>(out) + (long long)row * N;
@@ -340,29 +430,32 @@ k_rows_c2r4(RowJob<float> job, int nrows, int dq, void* __restrict__ out, signed
   }
 }
 
-// resident blocks: as many as fit on all SMs (each builds its tables once)
-template <class F> inline int row_grid(F fn, int threads, int smem, long long groups) {
-  int occ = 0;
+template <class F> inline void row_smem(F fn, int smem) {
   if (smem > 48 * 1024) ensure_smem_attr((const void*)fn, smem);
+}
+// resident blocks: as many as fit on all SMs (each builds its tables once)
+template <class F> inline int row_grid(F fn, int threads, int smem) {
+  int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess || occ < 1) {
     (void)cudaGetLastError();
     occ = 1;
   }
-  const long long most = (long long)occ * kNumSms;
-  return (int)(groups < most ? groups : most);
+  return occ * kNumSms;
 }
 
 template <int L>
 static void launch_rows_r2c(const RowJob<float>& job, int nbuf, int nrows, const float2* tw, cudaStream_t st) {
   using S = RowShape<L>;
-  static const int grid = row_grid(k_rows_r2c<L>, S::NT, S::SMEM, 1LL << 30);
+  row_smem(k_rows_r2c<L>, S::SMEM);
+  static const int grid = row_grid(k_rows_r2c<L>, S::NT, S::SMEM);
   const int groups = nrows / S::RPB * nbuf;
   k_rows_r2c<L><<<groups < grid ? groups : grid, S::NT, S::SMEM, st>>>(job, nrows, nbuf, tw + L, tw + 2 * L);
 }
 template <int L>
 static void launch_rows_c2r(const RowJob<float>& job, int nbuf, int nrows, const float2* tw, cudaStream_t st) {
   using S = RowShape<L>;
-  static const int grid = row_grid(k_rows_c2r<L>, S::NT, S::SMEM, 1LL << 30);
+  row_smem(k_rows_c2r<L>, S::SMEM);
+  static const int grid = row_grid(k_rows_c2r<L>, S::NT, S::SMEM);
   const int groups = nrows / S::RPB * nbuf;
   k_rows_c2r<L><<<groups < grid ? groups : grid, S::NT, S::SMEM, st>>>(job, nrows, nbuf, tw + L, tw + 2 * L);
 }
@@ -370,21 +463,18 @@ template <int L, int Q, bool H>
 static void launch_rows_c2r4_H(const RowJob<float>& job, int nrows, int dq, void* out, signed char* fexp, const float2* tw,
                                cudaStream_t st) {
   using S = RowShape<L>;
-  static const int grid = row_grid(k_rows_c2r4<L, Q, H>, S::NT, S::SMEM, 1LL << 30);
+  constexpr int smem = kRows4Smem<L, Q>;
+  row_smem(k_rows_c2r4<L, Q, H>, smem);
+  static const int grid = row_grid(k_rows_c2r4<L, Q, H>, S::NT, smem);
   const int groups = nrows / S::RPB;
-  k_rows_c2r4<L, Q, H><<<groups < grid ? groups : grid, S::NT, S::SMEM, st>>>(job, nrows, dq, out, fexp, tw + L,
+  k_rows_c2r4<L, Q, H><<<groups < grid ? groups : grid, S::NT, smem, st>>>(job, nrows, dq, out, fexp, tw + L,
                                                                             tw + 2 * L);
 }
-template <int L>
+template <int L, int Q>
 static void launch_rows_c2r4(const RowJob<float>& job, int nrows, int dq, void* out, signed char* fexp, const float2* tw,
                              cudaStream_t st) {
-  if (job.b[3].spec) {
-    if (fexp) launch_rows_c2r4_H<L, 4, true>(job, nrows, dq, out, fexp, tw, st);
-    else launch_rows_c2r4_H<L, 4, false>(job, nrows, dq, out, fexp, tw, st);
-  } else {
-    if (fexp) launch_rows_c2r4_H<L, 3, true>(job, nrows, dq, out, fexp, tw, st);
-    else launch_rows_c2r4_H<L, 3, false>(job, nrows, dq, out, fexp, tw, st);
-  }
+  if (fexp) launch_rows_c2r4_H<L, Q, true>(job, nrows, dq, out, fexp, tw, st);
+  else launch_rows_c2r4_H<L, Q, false>(job, nrows, dq, out, fexp, tw, st);
 }
 
 }  // namespace pmgb
