@@ -944,12 +944,20 @@ class Engine : public EngineBase {
   // (2^9 cells); the tile shape and threads per tile of the density-only deposit (forward)
   // and of the density + pi deposit (adjoint) are set separately (pm_tuning).
   int bin_setup() {
-    tune_.tile_log2_density[0] = 3; tune_.tile_log2_density[1] = 4; tune_.tile_log2_density[2] = 4;
-    tune_.tile_log2_adjoint[0] = 3; tune_.tile_log2_adjoint[1] = 4; tune_.tile_log2_adjoint[2] = 4;
+    // Deposit shapes.  Tiles long in x: the lattice neighbours of a warp spread over more rows'
+    // lines, and the write-out stores whole ones.  2^12 cells for the density, 2^11 with the pi sums
+    // (three blocks of 512 threads per SM); 2^10 where a mesh makes fewer than two such tiles per
+    // SM.  Deposit and x pass separately: fused, the four-quantity tile is one 128 KB block per SM
+    // whose phases cannot overlap (force VJP at 512^3 7.06 ms fused, 6.37 ms so; with the former
+    // tiles of 8 x 16 x 16 6.43 ms; at 1024^3 59.9, 51.3 and 51.9 ms).
+    const bool few = (long long)B_ * M_ < (2LL * nsm_ << 12);
+    const int td[3] = {few ? 2 : 3, few ? 2 : 4, few ? 6 : 5}, ta[3] = {2, few ? 2 : 3, 6};
+    for (int c = 0; c < 3; ++c) tune_.tile_log2_density[c] = td[c], tune_.tile_log2_adjoint[c] = ta[c];
     tune_.threads_density = 256;
     tune_.threads_adjoint = 512;
     tune_.tma_columns = 1;
-    tune_.fused_x = fused_rows<T>(nm_, 1) > 0 && !cfg_.fixed_state ? 3 : 0;
+    // (the density deposit of 128^3 meshes alone is faster fused: 145 against 147 us a force)
+    tune_.fused_x = nm_ == 128 && !cfg_.fixed_state ? 1 : 0;
     const BinGeo smallest = make_bin_geo(ilog2(nm_), 3, 3, 3);
     const long long maxbin = (long long)B_ * smallest.nkeys + 1;
     PMGB_RET(alloc(&bkeys_, (long long)B_ * N_));
