@@ -161,6 +161,13 @@ class Engine : public EngineBase {
     hf_ = cfg->half_force != 0 && sizeof(T) == 4;
     G_ = wave_grid((const void*)gather_adj_fn(), N_);
     Gf_ = wave_grid((const void*)gather_fwd_fn(), N_);
+    // The operators' gathers need few registers.  At 1024^3 (a 17 GB force mesh) more than two
+    // blocks per SM in flight span more pages than the address translation holds: force 28.9 ->
+    // 24.4 ms, force VJP 53.2 -> 47.2 ms with two; at 512^3 two are 1% slower than all that fit.
+    const long long two = nm_ >= 1024 ? 2LL * nsm_ * kPtclThreads : N_;
+    Gof_ = wave_grid((const void*)gather_fwd_fn<true>(), std::min(N_, two));
+    Goa_ = wave_grid((const void*)gather_adj_fn<true>(), std::min(N_, two));
+    Gpm_ = wave_grid((const void*)k_pi_max<T>, N_);
     Gc_ = wave_grid((const void*)k_bin_count<T>, N_);
     Gb1_ = wave_grid((const void*)k_bin_fill<T, 1>, N_);
     Gb4_ = wave_grid((const void*)k_bin_fill<T, 4>, N_);
@@ -406,32 +413,50 @@ class Engine : public EngineBase {
     counted_ = false;
     if (reinterpret_cast<uintptr_t>(dens) % (4 * sizeof(T))) return PM_ERR_ARG;   // vector stores
     have_fwd_ = false;
-    PMGB_CK(cudaMemcpyAsync(s_, disp, sizeof(T) * B_ * 3 * N_, cudaMemcpyDeviceToDevice, st_));
-    PMGB_RET(scatter(s_, nullptr, (T*)dens, M_));
+    const T* s = nullptr;
+    PMGB_RET(op_input(disp, dens, (long long)B_ * M_, nullptr, 0, s_, &s));
+    PMGB_RET(scatter(s, nullptr, (T*)dens, M_));
+    return PM_OK;
+  }
+
+  // The operators read the caller's particles where they lie: the deposit reads all of them
+  // before the gather writes a result.  Only inputs that overlap an output are copied first
+  // (into buf).
+  int op_input(const void* in, const void* out0, long long n0, const void* out1, long long n1, T* buf, const T** use) {
+    auto meets = [&](const void* out, long long n) {
+      const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out;
+      return out && a < b + sizeof(T) * n && b < a + sizeof(T) * B_ * 3 * N_;
+    };
+    *use = (const T*)in;
+    if (meets(out0, n0) || meets(out1, n1)) {
+      PMGB_CK(cudaMemcpyAsync(buf, in, sizeof(T) * B_ * 3 * N_, cudaMemcpyDeviceToDevice, st_));
+      *use = buf;
+    }
     return PM_OK;
   }
 
   int op_force(const void* disp, const void* pi, void* acc, void* alpha) override {
     counted_ = false;
     have_fwd_ = false;
-    PMGB_CK(cudaMemcpyAsync(s_, disp, sizeof(T) * B_ * 3 * N_, cudaMemcpyDeviceToDevice, st_));
-    const long long fis = 2 * spec_len_cx(nm_);
-    StepCoef<T> sc{zero_, zero_, zero_};
+    const long long pv = (long long)B_ * 3 * N_;
+    const T* s = nullptr;
+    PMGB_RET(op_input(disp, acc, pv, pi ? alpha : nullptr, pv, s_, &s));
     if (!pi) {
-      PMGB_RET(force_chain(s_, nullptr, false));
-      gather_fwd_fn()<<<dim3(Gf_, B_), kPtclThreads, 0, st_>>>(geo_, s_, p_, (T*)acc, fvec_, fexp_, sc, 0, 1, nullptr,
-                                                              nullptr, bg1_, nullptr, nullptr, nullptr, FixState<T>{});
+      PMGB_RET(force_chain(s, nullptr, false));
+      const auto fn = gather_fwd_fn<true>();
+      fn<<<dim3(Gof_, B_), kPtclThreads, 0, st_>>>(
+          geo_, const_cast<T*>(s), nullptr, (T*)acc, fvec_, fexp_, StepCoef<T>{}, 0, 1, nullptr, nullptr, bg1_, nullptr,
+          nullptr, nullptr, FixState<T>{});
     } else {
-      PMGB_CK(cudaMemcpyAsync(pi_, pi, sizeof(T) * B_ * 3 * N_, cudaMemcpyDeviceToDevice, st_));
+      const T* q = nullptr;
+      PMGB_RET(op_input(pi, acc, pv, alpha, pv, pi_, &q));
       PMGB_CK(cudaMemsetAsync(pimax_, 0, sizeof(unsigned) * 3 * B_, st_));
-      PMGB_CK(cudaMemsetAsync(xi_, 0, sizeof(T) * B_ * 3 * N_, st_));
-      // max|pi| through the adjoint init kernel with no cotangents except pi itself
-      k_adjoint_init<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, mass_, s_, nullptr, nullptr, (const T*)pi,
-                                                                xi_, pi_, pimax_);
-      PMGB_RET(force_chain(s_, pi_, false));
-      gather_adj_fn()<<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, mass_, s_, p_, xi_, pi_, (T*)acc, (T*)alpha,
-                                                              fvec_, fexp_, sc, 0, 1, nullptr, nullptr, nullptr, nullptr,
-                                                              nullptr, bg4_, nullptr, nullptr, FixState<T>{});
+      k_pi_max<T><<<dim3(Gpm_, B_), kPtclThreads, 0, st_>>>(q, N_, pimax_);
+      PMGB_RET(force_chain(s, q, false));
+      const auto fn = gather_adj_fn<true>();
+      fn<<<dim3(Goa_, B_), kPtclThreads, 0, st_>>>(
+          geo_, mass_, const_cast<T*>(s), nullptr, nullptr, const_cast<T*>(q), (T*)acc, (T*)alpha, fvec_, fexp_,
+          StepCoef<T>{}, 0, 1, nullptr, nullptr, nullptr, nullptr, nullptr, bg4_, nullptr, nullptr, FixState<T>{});
     }
     PMGB_CK(cudaGetLastError());
     return PM_OK;
@@ -830,8 +855,6 @@ class Engine : public EngineBase {
     PMGB_RET(upload(&gcoef_, gcoef));
     PMGB_RET(upload(&amp_, amp));
     PMGB_RET(upload(&hdl_, hdl));
-    std::vector<T> zero(B_, (T)0);
-    PMGB_RET(upload(&zero_, zero));
     if (cfg_.deconv) {
       std::vector<T> dt(nm_);
       for (int i = 0; i < nm_; ++i) {
@@ -1510,7 +1533,7 @@ class Engine : public EngineBase {
   pm_config cfg_{};
   cudaStream_t st_ = 0;
   int B_ = 1, np_ = 0, nm_ = 0, n_ = 0, lgN_ = 0, e_d_ = 0, G_ = 1, Gm_ = 1, Gz_ = 1, nck_ = 0, maxn2_ = 0;
-  int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1;   // grids of the particle loops
+  int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1;   // grids of the particle loops
 
   // Grid of a particle loop over `work` items: at most kMaxRedBlocks blocks, rounded down
   // to whole waves of the blocks the kernel keeps resident on all SMs.
@@ -1568,7 +1591,7 @@ class Engine : public EngineBase {
   double *wpa_ = nullptr, *wxp_ = nullptr, *dd1_ = nullptr, *dgd_ = nullptr, *dd2_ = nullptr, *dgd2_ = nullptr;
   T *s2_ = nullptr, *d2_ = nullptr, *gd2_ = nullptr, unit_ = 0;
   bool lpt2_ = false;
-  T *d1_ = nullptr, *gd_ = nullptr, *gcoef_ = nullptr, *amp_ = nullptr, *dtab_ = nullptr, *zero_ = nullptr;
+  T *d1_ = nullptr, *gd_ = nullptr, *gcoef_ = nullptr, *amp_ = nullptr, *dtab_ = nullptr;
   double* hdl_ = nullptr;
   C* tw_ = nullptr;
   unsigned* pimax_ = nullptr;
@@ -1583,16 +1606,16 @@ class Engine : public EngineBase {
   int nsm_ = 1;   // SM count
   bool hf_ = false;        // pm_config.half_force: the FP16 [cell][4] force mesh (FP32 path)
   int* fexp_ = nullptr;    // its int8 exponent quadruples, one int per mesh row [B][n][n]
-  // the gathers of the force mesh in its stored form
-  decltype(&k_gather_fwd<T, false>) gather_fwd_fn() const {
+  // the gathers of the force mesh in its stored form (OP: the operators' form)
+  template <bool OP = false> decltype(&k_gather_fwd<T, false, false>) gather_fwd_fn() const {
     if constexpr (sizeof(T) == 4)
-      if (hf_) return &k_gather_fwd<T, true>;
-    return &k_gather_fwd<T, false>;
+      if (hf_) return &k_gather_fwd<T, true, OP>;
+    return &k_gather_fwd<T, false, OP>;
   }
-  decltype(&k_gather_adj<T, false>) gather_adj_fn() const {
+  template <bool OP = false> decltype(&k_gather_adj<T, false, false>) gather_adj_fn() const {
     if constexpr (sizeof(T) == 4)
-      if (hf_) return &k_gather_adj<T, true>;
-    return &k_gather_adj<T, false>;
+      if (hf_) return &k_gather_adj<T, true, OP>;
+    return &k_gather_adj<T, false, OP>;
   }
   cudaStream_t cp_st_ = nullptr;                       // copy stream of pm_gradient's target
   cudaEvent_t cp_in_ = nullptr, cp_done_ = nullptr;     // its order after st_, its completion

@@ -324,7 +324,8 @@ struct StepCoef {  // per-instance coefficient tables [batch][n+1], indexed at s
 };
 
 // a = sum_g W f(g);  p += a kA;  (store p_j);  p += a kB;  (store s_j);  s += p dr
-template <typename T, bool H = false>
+// OP (the operator entry point): a into a_out and nothing else; reads the caller's s.
+template <typename T, bool H = false, bool OP = false>
 __global__ void __launch_bounds__(kPtclThreads)
 k_gather_fwd(Geo<T> g, T* __restrict__ s, T* __restrict__ p, T* __restrict__ a_out,
              const void* __restrict__ fvec, const int* __restrict__ fexp, StepCoef<T> sc, int j, int nstep1,
@@ -332,7 +333,8 @@ k_gather_fwd(Geo<T> g, T* __restrict__ s, T* __restrict__ p, T* __restrict__ a_o
              T* __restrict__ ck_p, BinGeo bg, unsigned* __restrict__ bcount, unsigned* __restrict__ bkeys,
              T* __restrict__ snap_p = nullptr, FixState<T> fx = FixState<T>{}) {
   const int b = blockIdx.y;
-  const T kA = sc.kA[b * nstep1 + j], kB = sc.kB[b * nstep1 + j], dr = sc.dr[b * nstep1 + j];
+  T kA = 0, kB = 0, dr = 0;
+  if constexpr (!OP) kA = sc.kA[b * nstep1 + j], kB = sc.kB[b * nstep1 + j], dr = sc.dr[b * nstep1 + j];
   T* sb = s + (long long)b * 3 * g.N;
   T* pb = p + (long long)b * 3 * g.N;
   // the displacement of the thread's next particle is read one iteration ahead, so that
@@ -348,7 +350,8 @@ k_gather_fwd(Geo<T> g, T* __restrict__ s, T* __restrict__ p, T* __restrict__ a_o
   for (; w < g.N; w += stride) {
     const long long i = particle_of(g, w);
     T sv[3] = {sn[0], sn[1], sn[2]};
-    T pv[3] = {pb[i], pb[g.N + i], pb[2 * g.N + i]};   // in flight with the corner loads
+    T pv[3] = {0, 0, 0};
+    if constexpr (!OP) pv[0] = pb[i], pv[1] = pb[g.N + i], pv[2] = pb[2 * g.N + i];   // in flight with the corner loads
     int cell[3];
     T t[3];
     cic_cell(g, i, sv, cell, t);
@@ -368,6 +371,11 @@ k_gather_fwd(Geo<T> g, T* __restrict__ s, T* __restrict__ p, T* __restrict__ a_o
       a[0] = fma_rn<T>(w, fv[d].x, a[0]);
       a[1] = fma_rn<T>(w, fv[d].y, a[1]);
       a[2] = fma_rn<T>(w, fv[d].z, a[2]);
+    }
+    if constexpr (OP) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) a_out[(long long)b * 3 * g.N + c * g.N + i] = a[c];
+      continue;
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -407,7 +415,8 @@ k_gather_fwd(Geo<T> g, T* __restrict__ s, T* __restrict__ p, T* __restrict__ a_o
 // Reverse step at force step j (Eq. 49): a_j = sum W f, alpha_j = sum grad W [pi.f + m psi];
 // p -= a K1_{j+1}; xi += alpha K1_{j+1}; (p := stored p_j); p -= a K2_j; xi += alpha K2_j;
 // s -= p D_j; pi += xi D_j; (s := stored s_{j-1}).  FP64 partials of pi.a and xi.p.
-template <typename T, bool H = false>
+// OP (the operator entry point): a and alpha into a_out and alpha_out and nothing else.
+template <typename T, bool H = false, bool OP = false>
 __global__ void __launch_bounds__(kPtclThreads)
 k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restrict__ xi, T* __restrict__ pi,
              T* __restrict__ a_out, T* __restrict__ alpha_out, const void* __restrict__ fvec,
@@ -418,7 +427,8 @@ k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restri
   __shared__ double shd[kPtclThreads / 32];
   __shared__ float shf[kPtclThreads / 32];
   const int b = blockIdx.y;
-  const T cA = sc.kA[b * nstep1 + j], cB = sc.kB[b * nstep1 + j], dr = sc.dr[b * nstep1 + j];
+  T cA = 0, cB = 0, dr = 0;
+  if constexpr (!OP) cA = sc.kA[b * nstep1 + j], cB = sc.kB[b * nstep1 + j], dr = sc.dr[b * nstep1 + j];
   const long long po = (long long)b * 3 * g.N;
   const T il = g.inv_l;
   KahanAcc<T> acc_pa, acc_xp;
@@ -430,8 +440,10 @@ k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restri
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       sv[c] = s[po + c * g.N + i];
-      pv[c] = p[po + c * g.N + i];
-      xv[c] = xi[po + c * g.N + i];
+      if constexpr (!OP) {
+        pv[c] = p[po + c * g.N + i];
+        xv[c] = xi[po + c * g.N + i];
+      }
       qv[c] = pi[po + c * g.N + i];
     }
     int cell[3];
@@ -454,6 +466,14 @@ k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restri
       al[0] += g0 * w1 * w2 * h;
       al[1] += w0 * g1 * w2 * h;
       al[2] += w0 * w1 * g2 * h;
+    }
+    if constexpr (OP) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        a_out[po + c * g.N + i] = a[c];
+        alpha_out[po + c * g.N + i] = al[c];
+      }
+      continue;
     }
     acc_pa.add(qv[0] * a[0] + qv[1] * a[1] + qv[2] * a[2]);
     long long W[3] = {0, 0, 0};
@@ -498,6 +518,7 @@ k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restri
     }
     if (bcount) count_bin(g, bg, i, sv, b, bcount, bkeys);   // bin for the previous step's deposit
   }
+  if constexpr (OP) return;
   const double spa = block_sum(acc_pa.value(), shd);
   const double sxp = block_sum(acc_xp.value(), shd);
   if (threadIdx.x == 0 && part_pa) {
@@ -510,6 +531,23 @@ k_gather_adj(Geo<T> g, T mass, T* __restrict__ s, T* __restrict__ p, T* __restri
       const float m = block_max(mx[c], shf);
       if (threadIdx.x == 0) atomicMax(pimax + c * gridDim.y + b, __float_as_uint(m));
     }
+  }
+}
+
+// max |pi_c| of every instance (layout [c][batch]), for the fixed-point exponents
+template <typename T>
+__global__ void __launch_bounds__(kPtclThreads)
+k_pi_max(const T* __restrict__ pi, long long N, unsigned* __restrict__ pimax) {
+  __shared__ float shf[kPtclThreads / 32];
+  const int b = blockIdx.y;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const T* q = pi + ((long long)b * 3 + c) * N;
+    float mx = 0.f;
+    for (long long i = blockIdx.x * (long long)kPtclThreads + threadIdx.x; i < N; i += (long long)gridDim.x * kPtclThreads)
+      mx = fmaxf(mx, abs_up<T>(q[i]));
+    const float m = block_max(mx, shf);
+    if (threadIdx.x == 0) atomicMax(pimax + c * gridDim.y + b, __float_as_uint(m));
   }
 }
 
