@@ -109,9 +109,10 @@ k_bin_fill(Geo<T> g, BinGeo bg, const T* __restrict__ s, const T* __restrict__ p
   }
 }
 
-// Exclusive scan of n counts in three launches: blocks of 2048 elements, the block totals
-// (one block), the add-back.  The scan also clears the counts for the next binning and
-// initialises the fill cursors.
+// Exclusive scan of n counts in two launches: blocks of 2048 elements, then the add-back, in
+// which every block sums the totals of the blocks before it (a third launch for that sum cost
+// more than the few thousand words it reads).  The scan also clears the counts for the next
+// binning and initialises the fill cursors.
 constexpr int kScanBlock = 2048;
 __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned* sh, unsigned* total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;   // 256 threads
@@ -162,34 +163,21 @@ static __global__ void __launch_bounds__(256) k_scan_blocks(unsigned* __restrict
   if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-static __global__ void __launch_bounds__(256) k_scan_sums(unsigned* __restrict__ sums, int nblocks) {
+static __global__ void __launch_bounds__(256) k_scan_add(unsigned* __restrict__ start, unsigned* __restrict__ cursor,
+                                                         const unsigned* __restrict__ sums, long long n) {
   __shared__ unsigned sh[8];
-  unsigned carry = 0;
-  for (int first = 0; first < nblocks; first += kScanBlock) {
-    const int base = first + threadIdx.x * 8;
-    unsigned v[8], tsum = 0;
+  constexpr int PER = kScanBlock / 256;
+  const long long base = (long long)blockIdx.x * kScanBlock + threadIdx.x;
+  unsigned v[PER], before = 0, total;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      v[k] = base + k < nblocks ? sums[base + k] : 0u;
-      tsum += v[k];
-    }
-    unsigned total;
-    unsigned run = carry + block_excl_scan(tsum, sh, &total);
+  for (int k = 0; k < PER; ++k) v[k] = base + 256 * k < n ? start[base + 256 * k] : 0u;
+  for (unsigned i = threadIdx.x; i < blockIdx.x; i += 256) before += sums[i];
+  block_excl_scan(before, sh, &total);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      if (base + k < nblocks) sums[base + k] = run;
-      run += v[k];
-    }
-    carry += total;
-  }
-}
-
-static __global__ void k_scan_add(unsigned* __restrict__ start, unsigned* __restrict__ cursor,
-                                  const unsigned* __restrict__ sums, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const unsigned v = start[i] + sums[i / kScanBlock];
-    start[i] = v;
-    cursor[i] = v;
+  for (int k = 0; k < PER; ++k) {
+    if (base + 256 * k >= n) break;
+    start[base + 256 * k] = v[k] + total;
+    cursor[base + 256 * k] = v[k] + total;
   }
 }
 

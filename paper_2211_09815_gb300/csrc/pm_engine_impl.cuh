@@ -186,6 +186,12 @@ class Engine : public EngineBase {
     PMGB_RET(alloc(&omega_, (long long)B_ * N_));
     // particle bins of the mesh-tile assignment (bin_kernels.cuh)
     PMGB_RET(bin_setup());
+    if (small_rule(1) || small_rule(4)) {
+      // sums of the small deposits, kept zero between calls
+      const long long n = (small_rule(4) ? 4 : 1) * (long long)B_ * M_;
+      PMGB_RET(alloc(&sacc_, n));
+      PMGB_CK(cudaMemsetAsync(sacc_, 0, sizeof(long long) * n, st_));
+    }
     for (int q = 0; q < 7; ++q) PMGB_RET(alloc(&spec_[q], sl));
     PMGB_RET(alloc(&dens_, (long long)B_ * M_));
     PMGB_RET(alloc(&fvec_, (long long)B_ * M_));
@@ -250,10 +256,11 @@ class Engine : public EngineBase {
       T* snap_p = (q >= 0 && snap_mom_) ? snap_mom_ + (long long)q * B_ * 3 * N_ : nullptr;
       prof_.begin(st_, P_GATHER_FWD, 1);
       // the bins of the next step's deposit are counted at the new positions
+      const bool count = j < n_ && !small_deposit(false);
       gather_fwd_fn()<<<dim3(Gf_, B_), kPtclThreads, 0, st_>>>(geo_, s_, p_, j == n_ ? a_ : nullptr, fvec_, fexp_, sc,
                                                               j, n_ + 1, cks, ckp, fused1_ ? bgf1_ : bg1_,
-                                                              j < n_ ? bcount_ : nullptr, bkeys_, snap_p, fx_);
-      counted_ = j < n_;
+                                                              count ? bcount_ : nullptr, bkeys_, snap_p, fx_);
+      counted_ = count;
       prof_.end(st_, P_GATHER_FWD);
       PMGB_CK(cudaGetLastError());
       // states observed between steps j and j + 1, from (s_{j+1}, p_{j+1/2})
@@ -354,12 +361,13 @@ class Engine : public EngineBase {
       StepCoef<T> sc{rkA_, rkB_, rdr_};
       double* ppa = part_ + (long long)(2 * j) * B_ * G_;
       double* pxp = part_ + (long long)(2 * j + 1) * B_ * G_;
+      const bool count = j > 0 && !small_deposit(true);
       prof_.begin(st_, P_GATHER_ADJ, 1);
       gather_adj_fn()<<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, mass_, s_, p_, xi_, pi_, vmom ? a_ : nullptr,
                                                               nullptr, fvec_, fexp_, sc, j, n_ + 1, ckp, cks, ppa, pxp,
                                                               pimax_, fused4_ ? bgf4_ : bg4_,
-                                                              j > 0 ? bcount_ : nullptr, bkeys_, fx_);
-      counted_ = j > 0;
+                                                              count ? bcount_ : nullptr, bkeys_, fx_);
+      counted_ = count;
       prof_.end(st_, P_GATHER_ADJ);
       PMGB_CK(cudaGetLastError());
       if (vmom) {
@@ -1036,6 +1044,7 @@ class Engine : public EngineBase {
     if (t->fused_x < 0 || t->fused_x > 3 || (t->fused_x && (fused_rows<T>(nm_, 1) == 0 || cfg_.fixed_state)))
       return PM_ERR_ARG;
     tune_ = *t;
+    tuned_ = true;
     apply_tuning();
     return PM_OK;
   }
@@ -1195,6 +1204,32 @@ class Engine : public EngineBase {
     }
     return tg;
   }
+  // Deposits of few particles (nq sums per cell) skip the bins: 64-bit global atomics into an
+  // integer mesh and one conversion, two launches instead of five.  The terms are rounded as
+  // in the tile deposit and the sums are exact, so the meshes are the same bit for bit.  The
+  // line: the atomics run at about 1e11 per second, 8 nq per particle, against some 20 us that
+  // the bins take at least; and the integer mesh is 8 nq bytes per cell, read and cleared.
+  // Shapes set by pm_set_tuning are taken as asked.
+  bool small_rule(int nq) const {
+    return nq * (long long)B_ * N_ <= (1LL << 18) && nq * (long long)B_ * M_ <= (1LL << 21);
+  }
+  bool small_deposit(bool pi) const { return !tuned_ && small_rule(pi ? 4 : 1); }
+  int scatter_small(const T* s, const T* pi, T* dout, long long dis, const SepTargets& tg) {
+    unsigned long long* acc = reinterpret_cast<unsigned long long*>(sacc_);
+    const dim3 gp((unsigned)std::min<long long>((N_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks), B_);
+    const dim3 gm((unsigned)std::min<long long>((M_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks), B_);
+    if (pi) {
+      k_scatter<T, 4><<<gp, kPtclThreads, 0, st_>>>(geo_, s, pi, acc, e_d_, e_pi_);
+      k_mesh_out<T, 4><<<gm, kPtclThreads, 0, st_>>>(sacc_, M_, e_d_, e_pi_, mass_, dout, dis, tg.p[0], tg.p[1], tg.p[2],
+                                                     tg.pis);
+    } else {
+      k_scatter<T, 1><<<gp, kPtclThreads, 0, st_>>>(geo_, s, nullptr, acc, e_d_, nullptr);
+      k_mesh_out<T, 1><<<gm, kPtclThreads, 0, st_>>>(sacc_, M_, e_d_, nullptr, mass_, dout, dis, nullptr, nullptr, nullptr,
+                                                     0);
+    }
+    PMGB_CK(cudaGetLastError());
+    return PM_OK;
+  }
   int scatter(const T* s, const T* pi, T* dout, long long dis, const FusedOut<T>* fo = nullptr,
               const SepTargets* tg = nullptr) {
     if (pi) {
@@ -1206,7 +1241,13 @@ class Engine : public EngineBase {
     }
     const bool pre = counted_;
     counted_ = false;
-    prof_.begin(st_, P_SCATTER, pre ? 5 : 6);
+    if (!fo && small_deposit(pi != nullptr)) {
+      prof_.begin(st_, P_SCATTER, 2);
+      PMGB_RET(scatter_small(s, pi, dout, dis, tg ? *tg : sep_targets(false)));
+      prof_.end(st_, P_SCATTER);
+      return PM_OK;
+    }
+    prof_.begin(st_, P_SCATTER, pre ? 4 : 5);
     if (fo)
       PMGB_RET(deposit(s, pi, nullptr, 0, pi ? bgf4_ : bgf1_, 0, pre, fo));
     else
@@ -1226,8 +1267,7 @@ class Engine : public EngineBase {
     const int nscan = (int)((nbin + kScanBlock - 1) / kScanBlock);
     if (!precounted) k_bin_count<T><<<dim3(Gc_, B_), kPtclThreads, 0, st_>>>(geo_, bg, s, bcount_, bkeys_);
     k_scan_blocks<<<nscan, 256, 0, st_>>>(bcount_, bstart_, bsums_, nbin);
-    k_scan_sums<<<1, 256, 0, st_>>>(bsums_, nscan);
-    k_scan_add<<<(int)std::min<long long>((nbin + 255) / 256, 4096), 256, 0, st_>>>(bstart_, bcursor_, bsums_, nbin);
+    k_scan_add<<<nscan, 256, 0, st_>>>(bstart_, bcursor_, bsums_, nbin);
     if (pi)
       k_bin_fill<T, 4><<<dim3(Gb4_, B_), kPtclThreads, 0, st_>>>(geo_, bg, s, pi, e_pi_, bkeys_, bcursor_, brec0_,
                                                                brec1_);
@@ -1276,7 +1316,7 @@ class Engine : public EngineBase {
   int force_chain(const T* s, const T* pi, bool keep_density) {
     // delta goes to the real view of spec_[0] (transformed in place) or, when the final
     // density is kept for the objective, to dens_
-    if (pi ? fused4_ : fused1_) {
+    if (!small_deposit(pi != nullptr) && (pi ? fused4_ : fused1_)) {
       // deposit and x pass in one kernel: delta (and pi_c) straight into the half spectra
       FusedOut<T> fo{};
       fo.spec[0] = spec_[0];
@@ -1581,6 +1621,8 @@ class Engine : public EngineBase {
   double fused_ms_[4] = {};   // autotuner: separate and fused deposit times (density, density + pi)   // forward (density) / adjoint (density + pi) deposit fused
   bool counted_ = false;   // the last gather counted the bins of the next deposit
   pm_tuning tune_{};
+  bool tuned_ = false;           // pm_set_tuning was called
+  long long* sacc_ = nullptr;    // integer mesh of the small deposits, zero between calls
   unsigned *bkeys_ = nullptr, *bcount_ = nullptr, *bstart_ = nullptr, *bcursor_ = nullptr, *bsums_ = nullptr;
   V4<T> *brec0_ = nullptr, *brec1_ = nullptr;
   C* spec_[7] = {};

@@ -196,6 +196,9 @@ template <> __device__ __forceinline__ float abs_up<double>(double v) { return _
 // ------------------------------------------------------------------------- scatter
 // NQ = 1: acc[cell] += W * 2^e_d (weights).  NQ = 4: acc is [cell][4] and receives the
 // weight and pi_c * W * 2^e_c (c = 0..2) in one 32-byte sector per cell.
+// (terms rounded as in the tile deposit; FP32 ones are at most 2^30 in magnitude, fixed_top)
+__device__ __forceinline__ unsigned long long term_fixed(float v) { return (unsigned long long)(long long)__float2int_rn(v); }
+__device__ __forceinline__ unsigned long long term_fixed(double v) { return (unsigned long long)__double2ll_rn(v); }
 template <typename T, int NQ>
 __global__ void __launch_bounds__(kPtclThreads)
 k_scatter(Geo<T> g, const T* __restrict__ s, const T* __restrict__ pi, unsigned long long* acc, int e_d,
@@ -203,13 +206,13 @@ k_scatter(Geo<T> g, const T* __restrict__ s, const T* __restrict__ pi, unsigned 
   const int b = blockIdx.y;
   const T* sb = s + (long long)b * 3 * g.N;
   const long long mo = (long long)b * g.M;
-  const T sd = (T)ldexp(1.0, e_d);
+  const T sd = pow2i<T>(e_d);
   T sp[3] = {0, 0, 0};
   const T* pb = nullptr;
   if constexpr (NQ == 4) {
     pb = pi + (long long)b * 3 * g.N;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) sp[c] = (T)ldexp(1.0, e_pi[c * gridDim.y + b]);
+    for (int c = 0; c < 3; ++c) sp[c] = pow2i<T>(e_pi[c * gridDim.y + b]);
   }
   for (long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x; w < g.N;
        w += (long long)gridDim.x * blockDim.x) {
@@ -229,13 +232,13 @@ k_scatter(Geo<T> g, const T* __restrict__ s, const T* __restrict__ pi, unsigned 
       const T w = ((d & 4) ? t[0] : (T)1 - t[0]) * ((d & 2) ? t[1] : (T)1 - t[1]) * ((d & 1) ? t[2] : (T)1 - t[2]);
       const long long idx = mo + corner_index(g, cell, d);
       if constexpr (NQ == 1) {
-        atomicAdd(acc + idx, (unsigned long long)to_fixed<T>(w * sd));
+        atomicAdd(acc + idx, term_fixed(w * sd));
       } else {
         unsigned long long* q = acc + 4 * idx;
-        atomicAdd(q, (unsigned long long)to_fixed<T>(w * sd));
-        atomicAdd(q + 1, (unsigned long long)to_fixed<T>(pv[0] * w));
-        atomicAdd(q + 2, (unsigned long long)to_fixed<T>(pv[1] * w));
-        atomicAdd(q + 3, (unsigned long long)to_fixed<T>(pv[2] * w));
+        atomicAdd(q, term_fixed(w * sd));
+        atomicAdd(q + 1, term_fixed(pv[0] * w));
+        atomicAdd(q + 2, term_fixed(pv[1] * w));
+        atomicAdd(q + 3, term_fixed(pv[2] * w));
       }
     }
   }
@@ -741,6 +744,39 @@ static __global__ void k_obs_theta(const double* __restrict__ sums, const double
   double acc = 0.0;
   for (int k = 0; k < nk; ++k) acc += w[(long long)k * batch + b] * sums[(long long)k * batch + b];
   theta[5 * b + 2] += acc;
+}
+
+// Real meshes from the sums of k_scatter<T, NQ>, the conversion of the tile deposit
+// (k_pull_scatter): delta = m acc 2^-e_d - 1 into dout (instance stride dis), pi_c = acc 2^-e_c
+// into p0..p2 (instance stride pis).  Leaves the sums zero for the next call.
+__device__ __forceinline__ float sum_to_real(long long v, float) { return ll2f_rn(v); }
+__device__ __forceinline__ double sum_to_real(long long v, double) { return (double)v; }
+template <typename T, int NQ>
+__global__ void __launch_bounds__(kPtclThreads)
+k_mesh_out(long long* __restrict__ acc, long long M, int e_d, const int* __restrict__ e_pi, T mass, T* __restrict__ dout,
+           long long dis, T* __restrict__ p0, T* __restrict__ p1, T* __restrict__ p2, long long pis) {
+  const int b = blockIdx.y;
+  const T md = mass * pow2i<T>(-e_d);
+  T mp[3] = {0, 0, 0};
+  if constexpr (NQ == 4) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) mp[c] = pow2i<T>(-e_pi[c * gridDim.y + b]);
+  }
+  for (long long i = blockIdx.x * (long long)kPtclThreads + threadIdx.x; i < M; i += (long long)gridDim.x * kPtclThreads) {
+    long long* a = acc + NQ * (b * M + i);
+    if constexpr (NQ == 1) {
+      dout[b * dis + i] = sum_to_real(a[0], (T)0) * md + (T)-1;
+      a[0] = 0;
+    } else {
+      longlong2* a2 = reinterpret_cast<longlong2*>(a);
+      const longlong2 v0 = a2[0], v1 = a2[1];
+      a2[0] = a2[1] = make_longlong2(0, 0);
+      dout[b * dis + i] = sum_to_real(v0.x, (T)0) * md + (T)-1;
+      p0[b * pis + i] = sum_to_real(v0.y, (T)0) * mp[0];
+      p1[b * pis + i] = sum_to_real(v1.x, (T)0) * mp[1];
+      p2[b * pis + i] = sum_to_real(v1.y, (T)0) * mp[2];
+    }
+  }
 }
 
 // delta = m acc 2^-e - 1 (no zeroing)
