@@ -102,6 +102,7 @@ class Engine : public EngineBase {
     if (cp_done_) cudaEventDestroy(cp_done_);
     if (graph_exec_) cudaGraphExecDestroy(graph_exec_);
     for (void* p : allocs_) cudaFree(p);
+    if (err_host_) cudaFreeHost(err_host_);
     live_bytes_add(-bytes_);
   }
 
@@ -121,11 +122,10 @@ class Engine : public EngineBase {
   }
   // PM_ERR_TIMEOUT if a bounded device wait gave up since the last check (clears the flag)
   int device_error() {
-    int e = 0;
-    PMGB_CK(cudaMemcpyAsync(&e, dev_err_, sizeof(int), cudaMemcpyDeviceToHost, st_));
     PMGB_CK(cudaStreamSynchronize(st_));
-    if (e) {
-      PMGB_CK(cudaMemsetAsync(dev_err_, 0, sizeof(int), st_));
+    volatile int* flag = err_host_;
+    if (*flag) {
+      *flag = 0;
       return PM_ERR_TIMEOUT;
     }
     return PM_OK;
@@ -221,8 +221,16 @@ class Engine : public EngineBase {
     tune_.tma_columns = (env && env[0] == '0' && spec_zb(nm_) <= 1) ? 0 : 1;
     apply_tuning();
     tune_.tma_columns = use_tma_ ? 1 : 0;
-    PMGB_RET(alloc(&dev_err_, 1));
-    PMGB_CK(cudaMemsetAsync(dev_err_, 0, sizeof(int), st_));
+    // the error flag lies in host memory that the device writes (only when a wait gives up), so
+    // that a check is the synchronisation alone, without a copy
+    if (!alloc_gate()) return PM_ERR_OOM;
+    if (cudaError_t e = cudaHostAlloc((void**)&err_host_, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable)) {
+      set_cuda_error(e);
+      cudaGetLastError();
+      return PM_ERR_OOM;
+    }
+    *err_host_ = 0;
+    PMGB_CK(cudaHostGetDevicePointer((void**)&dev_err_, err_host_, 0));
     if (tma_supported(nm_))
       for (int q = 0; q < 7; ++q) PMGB_RET(make_spec_tensor_maps<T>(nm_, B_, spec_[q], &tmy_[q], &tmz_[q]));
     PMGB_CK(cudaMemcpyAsync(omega_, omega, sizeof(T) * B_ * N_, cudaMemcpyDeviceToDevice, st_));
@@ -1661,7 +1669,8 @@ class Engine : public EngineBase {
   }
   cudaStream_t cp_st_ = nullptr;                       // copy stream of pm_gradient's target
   cudaEvent_t cp_in_ = nullptr, cp_done_ = nullptr;     // its order after st_, its completion
-  int* dev_err_ = nullptr;
+  int* err_host_ = nullptr;   // set by a bounded device wait that gave up (host memory)
+  int* dev_err_ = nullptr;    // its device address
   int first_wait_ = -1;   // spin limit of the TMA passes' first wait (test hook)
   CUtensorMap tmy_[7], tmz_[7];
 };
