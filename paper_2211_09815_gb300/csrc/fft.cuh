@@ -150,10 +150,20 @@ struct GlobalSeq {
   }
 };
 
+// Tiles whose rows take half of the 32 banks (64 bytes).  The first stage of a transform stores
+// rows R0 apart in one warp instruction, all on the same half of the banks.  Between the first
+// two stages such tiles keep row `row` at row ^ ((row / R0) & 1), which puts the rows of odd
+// butterflies on the other half; reads see neighbouring rows either way.
+template <class X, class = void> struct HalfBankRows { static constexpr bool value = false; };
+template <class X> struct HalfBankRows<X, decltype(void(X::kHalfBanks))> { static constexpr bool value = X::kHalfBanks; };
+
 // One Stockham radix-R stage over TC sequences of length L, NT threads.
 // NS = product of the radices already applied.  Loads all of the thread's inputs, syncs,
 // then stores, so source and destination may be the same shared-memory tile.
-template <typename T, int L, int TC, int NT, int R, int NS, int DIR, class Src, class Dst, class TW>
+// FLIP_ST: store (a first stage) into flipped rows; FLIP_LD: load rows flipped by blocks of
+// that many.
+template <typename T, int L, int TC, int NT, int R, int NS, int DIR, bool FLIP_ST = false, int FLIP_LD = 0, class Src,
+          class Dst, class TW>
 __device__ __forceinline__ void stage(const Src& src, const Dst& dst, const TW& tw) {
   using C = cx_t<T>;
   constexpr int ITEMS = TC * (L / R);
@@ -166,7 +176,15 @@ __device__ __forceinline__ void stage(const Src& src, const Dst& dst, const TW& 
     const int j = (threadIdx.x + i * NT) / TC;
     // rows j + r L/R: j < L/R, and L/R is a power of two, so the low four bits of j plus
     // those of r L/R never carry (a linear tile reads them at compile-time offsets)
-    if constexpr (IsLinear<Src>::value) {
+    if constexpr (FLIP_LD > 0) {
+      // block of row j + r L/R: j / FLIP_LD + r STEP
+      constexpr int STEP = (L / R) / FLIP_LD;
+      static_assert(STEP >= 1 && IsLinear<Src>::value, "flipped rows are loaded in whole blocks");
+      const C* const pe = src.ptr(j ^ ((j / FLIP_LD) & 1), c);
+      const C* const po = src.ptr(j ^ (((j / FLIP_LD) & 1) ^ 1), c);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[i][r] = ((r * STEP) & 1 ? po : pe)[Src::delta(r * (L / R)) * Src::kLD];
+    } else if constexpr (IsLinear<Src>::value) {
       const C* p = src.ptr(j, c);
 #pragma unroll
       for (int r = 0; r < R; ++r) v[i][r] = p[Src::delta(r * (L / R)) * Src::kLD];
@@ -188,7 +206,13 @@ __device__ __forceinline__ void stage(const Src& src, const Dst& dst, const TW& 
     const int jd = (j / NS) * NS * R + (j % NS);
     // rows jd + r NS: jd = (multiple of NS R) + (j mod NS); for NS >= 16 the step is a
     // multiple of 16, for NS < 16 (a power of two) the offsets stay inside the 16-row block
-    if constexpr (IsLinear<Dst>::value) {
+    if constexpr (FLIP_ST) {
+      static_assert(NS == 1 && R > 1 && IsLinear<Dst>::value, "flipped rows are stored by a first stage");
+      C* const pe = dst.ptr(jd + (j & 1), c);
+      C* const po = dst.ptr(jd - (j & 1), c);   // row jd + (r ^ 1) for odd r >= 1
+#pragma unroll
+      for (int r = 0; r < R; ++r) (r & 1 ? po : pe)[r * Dst::kLD] = v[i][r];
+    } else if constexpr (IsLinear<Dst>::value) {
       C* p = dst.ptr(jd, c);
 #pragma unroll
       for (int r = 0; r < R; ++r) p[Dst::delta(r * NS) * Dst::kLD] = v[i][r];
@@ -203,16 +227,17 @@ __device__ __forceinline__ void stage(const Src& src, const Dst& dst, const TW& 
 // radix plan (Plan<L> or Plan2<L>).
 template <typename T, int L, int TC, int NT, int DIR, class P = Plan<L>, class Src, class Mid, class Dst, class TW>
 __device__ __forceinline__ void fft_tile(const Src& src, const Mid& mid, const Dst& dst, const TW& tw) {
+  constexpr bool F = HalfBankRows<Mid>::value;
   if constexpr (P::S == 1) {
     stage<T, L, TC, NT, P::R0, 1, DIR>(src, dst, tw);
   } else if constexpr (P::S == 2) {
-    stage<T, L, TC, NT, P::R0, 1, DIR>(src, mid, tw);
+    stage<T, L, TC, NT, P::R0, 1, DIR, F>(src, mid, tw);
     __syncthreads();
-    stage<T, L, TC, NT, P::R1, P::R0, DIR>(mid, dst, tw);
+    stage<T, L, TC, NT, P::R1, P::R0, DIR, false, F ? P::R0 : 0>(mid, dst, tw);
   } else {
-    stage<T, L, TC, NT, P::R0, 1, DIR>(src, mid, tw);
+    stage<T, L, TC, NT, P::R0, 1, DIR, F>(src, mid, tw);
     __syncthreads();
-    stage<T, L, TC, NT, P::R1, P::R0, DIR>(mid, mid, tw);
+    stage<T, L, TC, NT, P::R1, P::R0, DIR, false, F ? P::R0 : 0>(mid, mid, tw);
     __syncthreads();
     stage<T, L, TC, NT, P::R2, P::R0 * P::R1, DIR>(mid, dst, tw);
   }

@@ -712,12 +712,12 @@ static void launch_fused_L(const ZJob<T>& job, bool adjoint, bool main, const cx
     launch_fused_S<T, L, false>(job, adjoint, main, tw, st);
 }
 
-template <typename T, int L> static int tiles_of() { return L * ((L / 2) / TmaTile<T, L>::TC); }
+template <typename T, int L, int KIND> static int tiles_of() { return L * ((L / 2) / TmaTile<T, L, KIND>::TC); }
 
 template <typename T, int L, int DIR, int KIND>
 static void launch_tma_L(const CUtensorMap* maps, const CUtensorMap* omaps, const TmaJob<T>& job, int tiles,
                          const cx_t<T>* tw, int nsm, cudaStream_t st) {
-  using TT = TmaTile<T, L, typename TmaPlanOf<T, L, KIND>::type>;
+  using TT = TmaTile<T, L, KIND>;
   TmaMaps m{}, om{};
   const int nomaps = (KIND == 1 || KIND == 3) ? 2 : ((KIND == 2 || KIND == 4) ? 1 : 0);
   for (int i = 0; i < nomaps; ++i) om.m[i] = omaps[i];
@@ -727,7 +727,7 @@ static void launch_tma_L(const CUtensorMap* maps, const CUtensorMap* omaps, cons
   auto fn = k_cols_tma<T, L, DIR, KIND>;
   ensure_smem_attr((const void*)fn, (int)sm);
   const int items = KIND == 0 ? job.nbuf * tiles : tiles;
-  const int grid = items < nsm ? items : nsm;
+  const int grid = items < TT::CTAS * nsm ? items : TT::CTAS * nsm;
   fn<<<grid, TT::NT, sm, st>>>(m, om, job, tiles, tw + L);
 }
 
@@ -751,9 +751,9 @@ int fft_cols_tma(int n, int batch, int dir, int zaxis, const CUtensorMap* maps, 
   job.err = wc.err;
   job.first_wait = wc.first_wait;
   if (dir < 0) {
-    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, -1, 0>(maps, nullptr, job, batch * tiles_of<T, LL>(), tw, nsm, st)));
+    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, -1, 0>(maps, nullptr, job, batch * tiles_of<T, LL, 0>(), tw, nsm, st)));
   } else {
-    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 0>(maps, nullptr, job, batch * tiles_of<T, LL>(), tw, nsm, st)));
+    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 0>(maps, nullptr, job, batch * tiles_of<T, LL, 0>(), tw, nsm, st)));
   }
   return PM_OK;
 }
@@ -769,7 +769,7 @@ int fft_ysplit_tma(int n, int batch, const CUtensorMap* umaps, cx_t<T>* u, cx_t<
   job.batch = batch;
   job.err = wc.err;
   job.first_wait = wc.first_wait;
-  PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 3>(umaps, umaps, job, batch * tiles_of<T, LL>(), tw, nsm, st)));
+  PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 3>(umaps, umaps, job, batch * tiles_of<T, LL, 3>(), tw, nsm, st)));
   return PM_OK;
 }
 
@@ -783,7 +783,7 @@ int fft_ymerge_tma(int n, int batch, const CUtensorMap* pmaps, cx_t<T>* p1, cons
   job.batch = batch;
   job.err = wc.err;
   job.first_wait = wc.first_wait;
-  PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, -1, 4>(pmaps, &pmaps[0], job, batch * tiles_of<T, LL>(), tw, nsm, st)));
+  PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, -1, 4>(pmaps, &pmaps[0], job, batch * tiles_of<T, LL, 4>(), tw, nsm, st)));
   return PM_OK;
 }
 
@@ -800,9 +800,9 @@ int fft_fused_tma(int n, bool adjoint, const CUtensorMap* maps, const CUtensorMa
   job.err = wc.err;
   job.first_wait = wc.first_wait;
   if (adjoint) {
-    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 2>(maps, omaps, job, zj.batch * tiles_of<T, LL>(), tw, nsm, st)));
+    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 2>(maps, omaps, job, zj.batch * tiles_of<T, LL, 2>(), tw, nsm, st)));
   } else {
-    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 1>(maps, omaps, job, zj.batch * tiles_of<T, LL>(), tw, nsm, st)));
+    PMGB_DISPATCH_TMA(n, (launch_tma_L<T, LL, +1, 1>(maps, omaps, job, zj.batch * tiles_of<T, LL, 1>(), tw, nsm, st)));
   }
   return PM_OK;
 }
@@ -810,7 +810,8 @@ int fft_fused_tma(int n, bool adjoint, const CUtensorMap* maps, const CUtensorMa
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).  The
 // spectrum main array is viewed as a 4-D tensor of int64 words: (kx words, y, z, batch).
 template <typename T, int L>
-static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap) {
+static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap,
+                       CUtensorMap* amap) {
   using Fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                           const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                           CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -823,7 +824,7 @@ static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* 
       return PM_ERR_CUDA;
     encode = (Fn)f;
   }
-  using TT = TmaTile<T, L>;
+  using TT = TmaTile<T, L, 0>;
   constexpr int eb = (int)sizeof(cx_t<T>);
   constexpr int ZB = TT::ZB;
   // main array as (kx words, z mod ZB, y, z / ZB, instance): row (z, y) at
@@ -835,18 +836,20 @@ static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* 
   const cuuint32_t ybox[5] = {(cuuint32_t)(TT::TC * TT::W), 1, (cuuint32_t)TT::RB, 1, 1};
   const cuuint32_t zbox[5] = {(cuuint32_t)(TT::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  const CUresult r1 = encode(ymap, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, (void*)buf, dims, strides, ybox, es,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  const CUresult r2 = encode(zmap, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, (void*)buf, dims, strides, zbox, es,
-                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return (r1 == CUDA_SUCCESS && r2 == CUDA_SUCCESS) ? PM_OK : PM_ERR_CUDA;
+  const cuuint32_t fbox[5] = {(cuuint32_t)(TmaTile<T, L, 1>::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
+  const cuuint32_t abox[5] = {(cuuint32_t)(TmaTile<T, L, 2>::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
+  auto make = [&](CUtensorMap* m, const cuuint32_t* box) {
+    return encode(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, (void*)buf, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  return make(ymap, ybox) && make(zmap, zbox) && make(fmap, fbox) && make(amap, abox) ? PM_OK : PM_ERR_CUDA;
 }
 
 template <typename T>
-int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap) {
-  PMGB_DISPATCH_TMA(n, return (make_maps_L<T, LL>(batch, buf, ymap, zmap)));
+int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap,
+                       CUtensorMap* amap) {
+  PMGB_DISPATCH_TMA(n, return (make_maps_L<T, LL>(batch, buf, ymap, zmap, fmap, amap)));
   return PM_ERR_ARG;
 }
 

@@ -117,6 +117,7 @@ struct DenseTile {
   __device__ __forceinline__ void st(int row, int c, C v) const { p[row * LD + c] = v; }
   static constexpr bool kLinear = true;
   static constexpr int kLD = LD;
+  static constexpr bool kHalfBanks = LD * sizeof(C) == 64;
   __device__ __forceinline__ C* ptr(int row, int c) const { return p + row * LD + c; }
   __host__ __device__ static constexpr int delta(int d) { return d; }
 };
@@ -124,8 +125,17 @@ struct DenseTile {
 // Tiles of the staged passes: 64 KB of TC columns (at least 128-byte rows of a TMA box for
 // L >= 512), transformed with the two-stage radix-32 plans at L = 512 and 1024, where a
 // third stage would add a read and a write of the whole tile in shared memory.
-template <typename T, int L> constexpr int tma_tc() {
-  return L >= 512 ? 65536 / (L * (int)sizeof(cx_t<T>)) : ColTile<T, L>::TC;
+//
+// The fused z passes, which compute three transforms per tile, take half of that and two CTAs per
+// SM up to L = 512 (KIND 1) and L = 256 (KIND 2), so that one's barriers and shared-memory
+// phases overlap the other's arithmetic: KIND 1 13.0 -> 10.8 us at 128^3, 56 -> 52 at 256^3, 452
+// -> 446 at 512^3; KIND 2 72 -> 68 us at 256^3, but 557 -> 570 at 512^3.  At L = 1024 half a tile
+// would be rows of 32 bytes.
+template <typename T, int L, int KIND> constexpr int tma_ctas() {
+  return (KIND == 1 && L <= 512) || (KIND == 2 && L <= 256) ? 2 : 1;
+}
+template <typename T, int L, int KIND> constexpr int tma_tc() {
+  return (L >= 512 ? 65536 / (L * (int)sizeof(cx_t<T>)) : ColTile<T, L>::TC) / tma_ctas<T, L, KIND>();
 }
 // Radix plan of a TMA column pass: the two-stage radix-32 plans, except for the fused
 // adjoint z pass (KIND 2), which takes the three-stage radix-16 plan where its thread count
@@ -136,12 +146,13 @@ template <typename T, int L> constexpr int tma_tc() {
 // without the hand-off and 11% slower with it, forward 16-8-8 into inverse 8-8-16), and
 // the y split and merge (KIND 3, 4) were 5% slower with radix 16.
 template <typename T, int L, int KIND> struct TmaPlanOf {
-  static constexpr bool kR16 = KIND == 2 && tma_tc<T, L>() * L / Plan<L>::RMAX <= 512;
+  static constexpr bool kR16 = KIND == 2 && tma_tc<T, L, KIND>() * L / Plan<L>::RMAX <= 512;
   using type = std::conditional_t<kR16, Plan<L>, Plan2<L>>;
 };
-template <typename T, int L, class PL = Plan2<L>> struct TmaTile {
-  using P = PL;
-  static constexpr int TC = tma_tc<T, L>();
+template <typename T, int L, int KIND> struct TmaTile {
+  using P = typename TmaPlanOf<T, L, KIND>::type;
+  static constexpr int CTAS = tma_ctas<T, L, KIND>();             // resident per SM
+  static constexpr int TC = tma_tc<T, L, KIND>();
   static constexpr int NT = TC * L / P::RMAX;
   static constexpr int LD = TC;
   static_assert(NT <= 512 && (L / 2) % TC == 0, "TMA tile shape");
@@ -245,11 +256,11 @@ struct YMergeDst {  // in place in the accumulator tile
 };
 
 template <typename T, int L, int DIR, int KIND>
-__global__ void __launch_bounds__(TmaTile<T, L, typename TmaPlanOf<T, L, KIND>::type>::NT, 1)
+__global__ void __launch_bounds__(TmaTile<T, L, KIND>::NT, TmaTile<T, L, KIND>::CTAS)
 k_cols_tma(const __grid_constant__ TmaMaps maps, const __grid_constant__ TmaMaps omaps,
            const __grid_constant__ TmaJob<T> job, int tiles_per_buf, const cx_t<T>* __restrict__ tw) {
   using C = cx_t<T>;
-  using TT = TmaTile<T, L, typename TmaPlanOf<T, L, KIND>::type>;
+  using TT = TmaTile<T, L, KIND>;
   constexpr int N = L;
   constexpr int NCG = (N / 2) / TT::TC;            // column groups per row of the main array
   constexpr int NL = (KIND == 2 || KIND == 4) ? 2 : 1;   // loads per work item
@@ -371,7 +382,8 @@ k_cols_tma(const __grid_constant__ TmaMaps maps, const __grid_constant__ TmaMaps
         // transforms start from registers instead of a shared-memory round trip
         constexpr int RA = TT::P::R0, RB = TT::P::R1, TC = TT::TC, NT = TT::NT;
         constexpr int PER = TC * (L / RB) / NT;
-        stage<T, L, TC, NT, RA, 1, -1>(t, t, stw);
+        constexpr bool F = HalfBankRows<DenseTile<C, TT::LD>>::value;   // flipped rows between stages
+        stage<T, L, TC, NT, RA, 1, -1, F>(t, t, stw);
         __syncthreads();
         C x[PER][RB];
         T gz[PER][RB];
@@ -379,7 +391,7 @@ k_cols_tma(const __grid_constant__ TmaMaps maps, const __grid_constant__ TmaMaps
         for (int i = 0; i < PER; ++i) {
           const int j = (threadIdx.x + i * NT) / TC;      // j < L / RB = RA
 #pragma unroll
-          for (int r = 0; r < RB; ++r) x[i][r] = cur[(j + r * RA) * TT::LD + c];
+          for (int r = 0; r < RB; ++r) x[i][r] = cur[((F ? j ^ (r & 1) : j) + r * RA) * TT::LD + c];
 #pragma unroll
           for (int r = 1; r < RB; ++r) x[i][r] = cmul(x[i][r], twiddle<-1>(stw, r * j));   // jm = j, L/(RA RB) = 1
           dft<RB, -1>(x[i]);                                // x[i][r] = X[j + RA r]
@@ -417,15 +429,15 @@ k_cols_tma(const __grid_constant__ TmaMaps maps, const __grid_constant__ TmaMaps
               y[r] = mode == 1 ? x[i][r] : cmake<C>(x[i][r].y * gz[i][r], -x[i][r].x * gz[i][r]);
             dft<RB, +1>(y);                                  // inverse stage 1 (NS = 1)
 #pragma unroll
-            for (int r = 0; r < RB; ++r) dst[(j * RB + r) * TT::LD + c] = y[r];
+            for (int r = 0; r < RB; ++r) dst[(j * RB + (F ? r ^ (j & 1) : r)) * TT::LD + c] = y[r];
           }
         }
         __syncthreads();
-        stage<T, L, TC, NT, RA, RB, +1>(wt, wt, stw);        // inverse stage 2 of the z force
+        stage<T, L, TC, NT, RA, RB, +1, false, F ? RB : 0>(wt, wt, stw);   // inverse stage 2 of the z force
         fence_proxy_async();
         __syncthreads();
         if (threadIdx.x == 0) store(&omaps.m[0], work, kxg, o, b);
-        stage<T, L, TC, NT, RA, RB, +1>(t, t, stw);          // and of U
+        stage<T, L, TC, NT, RA, RB, +1, false, F ? RB : 0>(t, t, stw);     // and of U
         fence_proxy_async();
         __syncthreads();
         if (threadIdx.x == 0) store(&omaps.m[1], cur, kxg, o, b);
