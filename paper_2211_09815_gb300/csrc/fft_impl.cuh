@@ -934,13 +934,15 @@ static void launch_c2r4_LQ(const RowJob<T>& job, int nrows, int dq, void* out, s
 template <typename T, int L>
 static void launch_c2r4_L(const RowJob<T>& job, int nrows, int dq, void* out, signed char* fexp, const cx_t<T>* tw,
                           cudaStream_t st) {
-  if constexpr (sizeof(T) == 4 && has_warp_rows(L)) {
-    if (!job.b[3].spec) return launch_rows_c2r4<L, 3>(job, nrows, dq, out, fexp, tw, st);
+  constexpr bool kRows = sizeof(T) == 4 && has_warp_rows(L);
+  if (job.b[3].spec) {
     // (four components of 128 points: 16 x 256^3 in 1.64 ms as tiles, 1.68 as rows)
-    if constexpr (L != 128) return launch_rows_c2r4<L, 4>(job, nrows, dq, out, fexp, tw, st);
+    if constexpr (kRows && L != 128) launch_rows_c2r4<L, 4>(job, nrows, dq, out, fexp, tw, st);
+    else launch_c2r4_LQ<T, L, 4>(job, nrows, dq, out, fexp, tw, st);
+  } else {
+    if constexpr (kRows) launch_rows_c2r4<L, 3>(job, nrows, dq, out, fexp, tw, st);
+    else launch_c2r4_LQ<T, L, 3>(job, nrows, dq, out, fexp, tw, st);
   }
-  if (job.b[3].spec) launch_c2r4_LQ<T, L, 4>(job, nrows, dq, out, fexp, tw, st);
-  else launch_c2r4_LQ<T, L, 3>(job, nrows, dq, out, fexp, tw, st);
 }
 
 template <typename T>
