@@ -171,6 +171,7 @@ class Engine : public EngineBase {
     Gc_ = wave_grid((const void*)k_bin_count<T>, N_);
     Gb1_ = wave_grid((const void*)k_bin_fill<T, 1>, N_);
     Gb4_ = wave_grid((const void*)k_bin_fill<T, 4>, N_);
+    Gi_ = (int)std::max<long long>(1, std::min<long long>((N_ + 255) / 256, 8LL * nsm_ / std::min(B_, 8)));   // lattice loops
     Gm_ = (int)std::min<long long>((M_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks);
     Gz_ = (int)std::min<long long>((spec_len_cx(np_) + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks);
     const long long pv = (long long)B_ * 3 * N_;
@@ -1437,12 +1438,12 @@ class Engine : public EngineBase {
     const long long lis = spec_len_cx(np_);
     // the lattice transforms use spec_[0..3] with the lattice instance stride
     PMGB_RET(lattice_r2c(omega_, N_, spec_[0]));
-    k_za_mul<T><<<dim3(256, B_), 256, 0, st_>>>(spec_[0], spec_[1], spec_[2], spec_[3], np_, amp_, maxn2_,
+    k_za_mul<T><<<dim3(Gi_, B_), 256, 0, st_>>>(spec_[0], spec_[1], spec_[2], spec_[3], np_, amp_, maxn2_,
                                                 inv_kfp_, lis, (T)0);
     PMGB_CK(cudaGetLastError());
     C* bufs[3] = {spec_[1], spec_[2], spec_[3]};
     PMGB_RET(lattice_c2r(bufs, 3));
-    k_ic_state<T><<<dim3(256, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, d1_, gd_, s1_, s_, p_);
+    k_ic_state<T><<<dim3(Gi_, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, d1_, gd_, s1_, s_, p_);
     PMGB_CK(cudaGetLastError());
     if (lpt2_) PMGB_RET(lpt2_state());
     if (fx_.u) {
@@ -1460,19 +1461,19 @@ class Engine : public EngineBase {
     const long long lis = spec_len_cx(np_);
     C* h[3] = {spec_[1], spec_[2], spec_[3]};
     for (int g = 0; g < 2; ++g) {
-      k_lpt_hess<T><<<dim3(256, B_), 256, 0, st_>>>(spec_[0], h[0], h[1], h[2], np_, amp_, maxn2_, lis, g);
+      k_lpt_hess<T><<<dim3(Gi_, B_), 256, 0, st_>>>(spec_[0], h[0], h[1], h[2], np_, amp_, maxn2_, lis, g);
       PMGB_CK(cudaGetLastError());
       PMGB_RET(lattice_c2r(h, 3));
-      k_lpt_source<T><<<dim3(256, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, rmesh(4), 2 * lis,
+      k_lpt_source<T><<<dim3(Gi_, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, rmesh(4), 2 * lis,
                                                       g);
       PMGB_CK(cudaGetLastError());
     }
     PMGB_RET(lattice_r2c(rmesh(4), 2 * lis, spec_[4]));
-    k_za_mul<T><<<dim3(256, B_), 256, 0, st_>>>(spec_[4], h[0], h[1], h[2], np_, nullptr, maxn2_, inv_kfp_, lis,
+    k_za_mul<T><<<dim3(Gi_, B_), 256, 0, st_>>>(spec_[4], h[0], h[1], h[2], np_, nullptr, maxn2_, inv_kfp_, lis,
                                                 unit_);
     PMGB_CK(cudaGetLastError());
     PMGB_RET(lattice_c2r(h, 3));
-    k_ic_state2<T><<<dim3(256, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, d2_, gd2_, s2_, s_,
+    k_ic_state2<T><<<dim3(Gi_, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, d2_, gd2_, s2_, s_,
                                                    p_);
     PMGB_CK(cudaGetLastError());
     return PM_OK;
@@ -1506,10 +1507,10 @@ class Engine : public EngineBase {
     PMGB_RET(lattice_c2r(sb, 1));
     C* h[3] = {spec_[1], spec_[2], spec_[3]};
     for (int g = 0; g < 2; ++g) {
-      k_lpt_hess<T><<<dim3(256, B_), 256, 0, st_>>>(spec_[0], h[0], h[1], h[2], np_, amp_, maxn2_, lis, g);
+      k_lpt_hess<T><<<dim3(Gi_, B_), 256, 0, st_>>>(spec_[0], h[0], h[1], h[2], np_, amp_, maxn2_, lis, g);
       PMGB_CK(cudaGetLastError());
       PMGB_RET(lattice_c2r(h, 3));
-      k_lpt_source_adj<T><<<dim3(256, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, rmesh(4),
+      k_lpt_source_adj<T><<<dim3(Gi_, B_), 256, 0, st_>>>(rmesh(1), rmesh(2), rmesh(3), 2 * lis, N_, rmesh(4),
                                                           2 * lis, g);
       PMGB_CK(cudaGetLastError());
       RowJob<T> jh{};
@@ -1518,7 +1519,7 @@ class Engine : public EngineBase {
       PMGB_CK(cudaGetLastError());
       PMGB_RET(cols(np_, -1, false, h, 3, false));
       PMGB_RET(cols(np_, -1, true, h, 3, false));
-      k_lpt_hess_adj<T><<<dim3(256, B_), 256, 0, st_>>>(spec_[1], spec_[2], spec_[3], spec_[5], np_, amp_, maxn2_,
+      k_lpt_hess_adj<T><<<dim3(Gi_, B_), 256, 0, st_>>>(spec_[1], spec_[2], spec_[3], spec_[5], np_, amp_, maxn2_,
                                                         lis, g);
       PMGB_CK(cudaGetLastError());
     }
@@ -1581,7 +1582,7 @@ class Engine : public EngineBase {
   pm_config cfg_{};
   cudaStream_t st_ = 0;
   int B_ = 1, np_ = 0, nm_ = 0, n_ = 0, lgN_ = 0, e_d_ = 0, G_ = 1, Gm_ = 1, Gz_ = 1, nck_ = 0, maxn2_ = 0;
-  int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1;   // grids of the particle loops
+  int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1, Gi_ = 1;   // grids of the particle loops
 
   // Grid of a particle loop over `work` items: at most kMaxRedBlocks blocks, rounded down
   // to whole waves of the blocks the kernel keeps resident on all SMs.

@@ -807,32 +807,18 @@ k_mse(const T* __restrict__ dens, const T* __restrict__ tgt, T* __restrict__ gra
 }
 
 // ------------------------------------------------------------------ lattice spectra
-// Mode (i0, i1, kx) of an n^3 half spectrum from a flat index over main + side (main rows
-// z-blocked by zb, spec_row).
-struct Mode { int f0, f1, f2; long long off; };
-__device__ __forceinline__ Mode mode_of(long long u, int n, int zb = 1) {
-  Mode m;
+// Mode (i0, i1, kx) of an n^3 half spectrum from a flat index over main + side (n a power of
+// two: shifts; 64-bit divisions took longer than the rest of the lattice kernels).
+struct Mode { int f0, f1, f2; };
+__device__ __forceinline__ Mode mode_of(long long u, int n) {
+  const int lg = 31 - __clz(n);
   const long long main = (long long)n * n * (n / 2);
-  if (u < main) {
-    const int kx = (int)(u % (n / 2));
-    const long long t = u / (n / 2);
-    if (zb <= 1) {
-      m.f1 = freq_of((int)(t % n), n);
-      m.f0 = freq_of((int)(t / n), n);
-    } else {
-      const int zlo = (int)(t % zb);
-      const long long t2 = t / zb;
-      m.f1 = freq_of((int)(t2 % n), n);
-      m.f0 = freq_of((int)(t2 / n) * zb + zlo, n);
-    }
-    m.f2 = kx;
-  } else {
-    const long long v = u - main;
-    m.f1 = freq_of((int)(v % n), n);
-    m.f0 = freq_of((int)(v / n), n);
-    m.f2 = n / 2;
-  }
-  m.off = u;
+  const bool in = u < main;
+  const long long t = in ? u >> (lg - 1) : u - main;
+  Mode m;
+  m.f1 = freq_of((int)t & (n - 1), n);
+  m.f0 = freq_of((int)(t >> lg), n);
+  m.f2 = in ? (int)u & (n / 2 - 1) : n / 2;
   return m;
 }
 __device__ __forceinline__ int nyq_zero(int f, int n, bool last) { return last ? (f == n / 2 ? 0 : f) : (f == -n / 2 ? 0 : f); }
@@ -1013,14 +999,17 @@ __global__ void k_ic_state2(const T* __restrict__ r0, const T* __restrict__ r1, 
                             T* s, T* p) {
   const int b = blockIdx.y;
   const T* rs[3] = {r0 + b * ris, r1 + b * ris, r2 + b * ris};
+  const T d = d2[b], gd = gd2[b];
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const long long o = (long long)b * 3 * N + i;
+    T v[3], sv[3], pv[3];   // every load before the first store
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v[c] = rs[c][i], sv[c] = s[o + c * N], pv[c] = p[o + c * N];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const T v = rs[c][i];
-      const long long o = (long long)b * 3 * N + c * N + i;
-      s2[o] = v;
-      s[o] = s[o] + d2[b] * v;
-      p[o] = p[o] + gd2[b] * v;
+      s2[o + c * N] = v[c];
+      s[o + c * N] = sv[c] + d * v[c];
+      p[o + c * N] = pv[c] + gd * v[c];
     }
   }
 }
@@ -1032,13 +1021,13 @@ __global__ void k_ic_state(const T* __restrict__ r0, const T* __restrict__ r1, c
   const int b = blockIdx.y;
   const T* rs[3] = {r0 + b * ris, r1 + b * ris, r2 + b * ris};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const T v[3] = {rs[0][i], rs[1][i], rs[2][i]};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const T v = rs[c][i];
       const long long o = (long long)b * 3 * N + c * N + i;
-      if (s1) s1[o] = v;
-      if (s) s[o] = d1[b] * v;
-      if (p) p[o] = gd[b] * v;
+      if (s1) s1[o] = v[c];
+      if (s) s[o] = d1[b] * v[c];
+      if (p) p[o] = gd[b] * v[c];
     }
   }
 }
