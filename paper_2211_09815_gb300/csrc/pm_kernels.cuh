@@ -1131,7 +1131,7 @@ static __global__ void k_final_theta(ThetaIn in, double* out) {
 // memory where the bin changes, and a block adds its bins to the global ones once.  FP32
 // spectra are squared and rounded to fixed point in error-free FP32 pairs, not on the slow
 // FP64 pipe.  Measured at 256^3 (67 MB spectrum): one global atomic per mode and FP64
-// arithmetic took 667 + 800 us for the two passes, these 19 + 29 us.
+// arithmetic took 667 + 800 us for the two passes, these 19 + 29 us; the cotangent 60, now 25 us.
 constexpr int kPowerMaxBins = 512;
 constexpr int kPowerThreads = 256;
 
@@ -1164,6 +1164,18 @@ inline PowerRuns power_runs(int n, int lzb) {
   r.lglen = r.lgn - 1 < 3 ? r.lgn - 1 : 3;
   r.count = ((long long)n * n * (n / 2)) >> r.lglen;
   return r;
+}
+
+// a run of 4 or 8 modes, in pairs (16-byte loads for FP32: a lane's run is 64 bytes)
+template <typename C> struct alignas(2 * sizeof(C)) ModePair { C a, b; };
+template <typename C> __device__ __forceinline__ void load_run(const C* p, int lglen, C (&v)[8]) {
+  const ModePair<C>* q = reinterpret_cast<const ModePair<C>*>(p);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (2 * k < (1 << lglen)) {
+      const ModePair<C> m = q[k];
+      v[2 * k] = m.a, v[2 * k + 1] = m.b;
+    }
 }
 
 // an upper bound of w |v|^2 as a float, w = 2^lw
@@ -1219,9 +1231,7 @@ k_power_max(const cx_t<T>* __restrict__ spec, PowerRuns pr, long long is, int nb
     int bin = isqrt_floor(n01 + kx * kx);
     if (bin >= nb) continue;                             // |n| only grows along the run
     cx_t<T> v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < (1 << pr.lglen)) v[k] = p[k];
+    load_run(p, pr.lglen, v);
     float m = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -1265,9 +1275,7 @@ k_power_acc(const cx_t<T>* __restrict__ spec, PowerRuns pr, long long is, int nb
     int bin = isqrt_floor(n01 + kx * kx);
     if (bin >= nb) continue;
     cx_t<T> v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < (1 << pr.lglen)) v[k] = p[k];
+    load_run(p, pr.lglen, v);
     long long a = 0;
     int e = se[bin];
 #pragma unroll
@@ -1387,9 +1395,7 @@ k_power_grad(cx_t<T>* spec, PowerRuns pr, long long is, int nb, const double* __
     cx_t<T>* p = sp + pr.at(u, kx, n01);
     int bin = isqrt_floor(n01 + kx * kx);
     cx_t<T> v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < (1 << pr.lglen)) v[k] = p[k];
+    load_run(p, pr.lglen, v);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (k >= (1 << pr.lglen)) break;
@@ -1398,8 +1404,10 @@ k_power_grad(cx_t<T>* spec, PowerRuns pr, long long is, int nb, const double* __
       const T f = bin < nb ? sg[bin] : (T)0;
       v[k].x *= f;
       v[k].y *= f;
-      p[k] = v[k];
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (2 * k < (1 << pr.lglen)) reinterpret_cast<ModePair<cx_t<T>>*>(p)[k] = ModePair<cx_t<T>>{v[2 * k], v[2 * k + 1]};
   }
   const long long side = (long long)n * n * (n / 2);
   for (int i = blockIdx.x * kPowerThreads + threadIdx.x; i < n * n; i += gridDim.x * kPowerThreads) {
