@@ -279,8 +279,10 @@ k_cols_tma(const __grid_constant__ TmaMaps maps, const __grid_constant__ TmaMaps
   constexpr int NCG = (N / 2) / TT::TC;            // column groups per row of the main array
   constexpr int NL = (KIND == 2 || KIND == 4) ? 2 : 1;   // loads per work item
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // TMA destinations must be 128-byte aligned: round the dynamic base up (1 KiB slack)
-  C* ring0 = reinterpret_cast<C*>((reinterpret_cast<unsigned long long>(smem_raw) + 1023ull) & ~1023ull);
+  // TMA destinations must be 128-byte aligned: round the dynamic base up (1 KiB slack).  By an
+  // offset, not through an integer address: the pointer stays one into shared memory for the
+  // compiler, and the tile accesses shared-memory instructions instead of generic ones.
+  C* ring0 = reinterpret_cast<C*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
   // ring slots of the prefetched tiles: three for the plain passes (no work tile), two
   // and a work tile for the others
   constexpr int NSLOT = KIND == 0 ? 3 : 2;
