@@ -164,9 +164,9 @@ class Engine : public EngineBase {
     // The operators' gathers need few registers.  At 1024^3 (a 17 GB force mesh) more than two
     // blocks per SM in flight span more pages than the address translation holds: force 28.9 ->
     // 24.4 ms, force VJP 53.2 -> 47.2 ms with two; at 512^3 two are 1% slower than all that fit.
-    const long long two = nm_ >= 1024 ? 2LL * nsm_ * kPtclThreads : N_;
-    Gof_ = wave_grid((const void*)gather_fwd_fn<true>(), std::min(N_, two));
-    Goa_ = wave_grid((const void*)gather_adj_fn<true>(), std::min(N_, two));
+    const int most = nm_ >= 1024 ? 2 * nsm_ : kMaxRedBlocks;
+    Gof_ = std::min(most, wave_grid((const void*)gather_fwd_fn<true>(), N_));
+    Goa_ = std::min(most, wave_grid((const void*)gather_adj_fn<true>(), N_));
     Gpm_ = wave_grid((const void*)k_pi_max<T>, N_);
     Gc_ = wave_grid((const void*)k_bin_count<T>, N_);
     Gb1_ = wave_grid((const void*)k_bin_fill<T, 1>, N_);
@@ -1584,8 +1584,14 @@ class Engine : public EngineBase {
   int B_ = 1, np_ = 0, nm_ = 0, n_ = 0, lgN_ = 0, e_d_ = 0, G_ = 1, Gm_ = 1, Gz_ = 1, nck_ = 0, maxn2_ = 0;
   int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1, Gi_ = 1;   // grids of the particle loops
 
-  // Grid of a particle loop over `work` items: at most kMaxRedBlocks blocks, rounded down
-  // to whole waves of the blocks the kernel keeps resident on all SMs.
+  // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
+  // resident on all SMs, of a batch of small instances fewer, eight particles to a thread.
+  // (Several whole waves scatter the blocks in flight over the lattice as they drift apart:
+  // adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3 and 1024^3, with one 102, 742
+  // and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470 with one.  The sums at the
+  // end of an adjoint block cost as much as several particles: 8 x 64^3 particles 177 us with one
+  // to a thread, 91 with 27.  But one wave over 16 instances of 128^3 mixes their meshes in the L2:
+  // 1204 us against 836 with one wave for each.)
   int wave_grid(const void* fn, long long work) const {
     const long long need = (work + kPtclThreads - 1) / kPtclThreads;
     int occ = 0;
@@ -1593,9 +1599,8 @@ class Engine : public EngineBase {
       (void)cudaGetLastError();
       occ = 1;
     }
-    const long long wave = (long long)occ * nsm_;
-    const long long cap = wave >= kMaxRedBlocks ? kMaxRedBlocks : (kMaxRedBlocks / wave) * wave;
-    return (int)std::max<long long>(1, std::min(need, cap));
+    const long long wave = std::min<long long>((long long)occ * nsm_, kMaxRedBlocks);
+    return (int)std::max<long long>(1, std::min(need, std::min(wave, std::max(wave / B_, need / 8))));
   }
   long long N_ = 0, M_ = 0, bytes_ = 0;
   T mass_ = 1, inv_kfp_ = 1;
