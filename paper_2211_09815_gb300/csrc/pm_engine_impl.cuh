@@ -1585,7 +1585,7 @@ class Engine : public EngineBase {
   int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1, Gi_ = 1;   // grids of the particle loops
 
   // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
-  // resident on all SMs, of a batch of small instances fewer, eight particles to a thread.
+  // resident on all SMs, of a batch of small instances fewer, up to 16 particles to a thread.
   // (Several whole waves scatter the blocks in flight over the lattice as they drift apart:
   // adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3 and 1024^3, with one 102, 742
   // and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470 with one.  The sums at the
@@ -1600,7 +1600,7 @@ class Engine : public EngineBase {
       occ = 1;
     }
     const long long wave = std::min<long long>((long long)occ * nsm_, kMaxRedBlocks);
-    return (int)std::max<long long>(1, std::min(need, std::min(wave, std::max(wave / B_, need / 8))));
+    return (int)std::max<long long>(1, std::min(need, std::min(wave, std::max(wave / B_, need / 16))));
   }
   long long N_ = 0, M_ = 0, bytes_ = 0;
   T mass_ = 1, inv_kfp_ = 1;
