@@ -11,7 +11,7 @@ template int fft_cols_tma<float>(int, int, int, int, const CUtensorMap*, cx_t<fl
                                 const WaitCtl&, int, cudaStream_t);
 template int fft_fused_tma<float>(int, bool, const CUtensorMap*, const CUtensorMap*, const ZJob<float>&, const cx_t<float>*, const WaitCtl&, int,
                                  cudaStream_t);
-template int make_spec_tensor_maps<float>(int, int, cx_t<float>*, CUtensorMap*, CUtensorMap*, CUtensorMap*, CUtensorMap*);
+template int make_spec_tensor_maps<float>(int, int, cx_t<float>*, CUtensorMap*, CUtensorMap*, CUtensorMap*);
 template int fft_x_c2r4<float>(int, const RowJob<float>&, int, int, void*, signed char*, const cx_t<float>*, cudaStream_t);
 template int fft_cols_split<float>(int, const SeqMap&, const SeqMap&, cx_t<float>*, cx_t<float>*, const cx_t<float>*,
                                    cudaStream_t);

@@ -11,7 +11,7 @@ template int fft_cols_tma<double>(int, int, int, int, const CUtensorMap*, cx_t<d
                                 const WaitCtl&, int, cudaStream_t);
 template int fft_fused_tma<double>(int, bool, const CUtensorMap*, const CUtensorMap*, const ZJob<double>&, const cx_t<double>*, const WaitCtl&, int,
                                  cudaStream_t);
-template int make_spec_tensor_maps<double>(int, int, cx_t<double>*, CUtensorMap*, CUtensorMap*, CUtensorMap*, CUtensorMap*);
+template int make_spec_tensor_maps<double>(int, int, cx_t<double>*, CUtensorMap*, CUtensorMap*, CUtensorMap*);
 template int fft_x_c2r4<double>(int, const RowJob<double>&, int, int, void*, signed char*, const cx_t<double>*, cudaStream_t);
 template int fft_cols_split<double>(int, const SeqMap&, const SeqMap&, cx_t<double>*, cx_t<double>*, const cx_t<double>*,
                                    cudaStream_t);

@@ -810,8 +810,7 @@ int fft_fused_tma(int n, bool adjoint, const CUtensorMap* maps, const CUtensorMa
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no libcuda link).  The
 // spectrum main array is viewed as a 4-D tensor of int64 words: (kx words, y, z, batch).
 template <typename T, int L>
-static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap,
-                       CUtensorMap* amap) {
+static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap) {
   using Fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                           const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                           CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -837,19 +836,18 @@ static int make_maps_L(int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* 
   const cuuint32_t zbox[5] = {(cuuint32_t)(TT::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   const cuuint32_t fbox[5] = {(cuuint32_t)(TmaTile<T, L, 1>::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
-  const cuuint32_t abox[5] = {(cuuint32_t)(TmaTile<T, L, 2>::TC * TT::W), (cuuint32_t)ZB, 1, (cuuint32_t)(TT::RB / ZB), 1};
+  static_assert(TmaTile<T, L, 1>::TC == TmaTile<T, L, 2>::TC, "the fused z passes share a map");
   auto make = [&](CUtensorMap* m, const cuuint32_t* box) {
     return encode(m, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, (void*)buf, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   };
-  return make(ymap, ybox) && make(zmap, zbox) && make(fmap, fbox) && make(amap, abox) ? PM_OK : PM_ERR_CUDA;
+  return make(ymap, ybox) && make(zmap, zbox) && make(fmap, fbox) ? PM_OK : PM_ERR_CUDA;
 }
 
 template <typename T>
-int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap,
-                       CUtensorMap* amap) {
-  PMGB_DISPATCH_TMA(n, return (make_maps_L<T, LL>(batch, buf, ymap, zmap, fmap, amap)));
+int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap) {
+  PMGB_DISPATCH_TMA(n, return (make_maps_L<T, LL>(batch, buf, ymap, zmap, fmap)));
   return PM_ERR_ARG;
 }
 

@@ -127,13 +127,10 @@ struct DenseTile {
 // third stage would add a read and a write of the whole tile in shared memory.
 //
 // The fused z passes, which compute three transforms per tile, take half of that and two CTAs per
-// SM up to L = 512 (KIND 1) and L = 256 (KIND 2), so that one's barriers and shared-memory
-// phases overlap the other's arithmetic: KIND 1 13.0 -> 10.8 us at 128^3, 56 -> 52 at 256^3, 452
-// -> 446 at 512^3; KIND 2 72 -> 68 us at 256^3, but 557 -> 570 at 512^3.  At L = 1024 half a tile
-// would be rows of 32 bytes.
-template <typename T, int L, int KIND> constexpr int tma_ctas() {
-  return (KIND == 1 && L <= 512) || (KIND == 2 && L <= 256) ? 2 : 1;
-}
+// SM up to L = 256, so that one's barriers and shared-memory phases overlap the other's
+// arithmetic (16 x 256^3: KIND 1 608 -> 580 us, KIND 2 847 -> 728; at 512^3 KIND 1 366 -> 372, KIND 2
+// 417 -> 434; at L = 1024 half a tile would be rows of 32 bytes).
+template <typename T, int L, int KIND> constexpr int tma_ctas() { return (KIND == 1 || KIND == 2) && L <= 256 ? 2 : 1; }
 template <typename T, int L, int KIND> constexpr int tma_tc() {
   return (L >= 512 ? 65536 / (L * (int)sizeof(cx_t<T>)) : ColTile<T, L>::TC) / tma_ctas<T, L, KIND>();
 }

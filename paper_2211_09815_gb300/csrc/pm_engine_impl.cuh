@@ -233,7 +233,7 @@ class Engine : public EngineBase {
     *err_host_ = 0;
     PMGB_CK(cudaHostGetDevicePointer((void**)&dev_err_, err_host_, 0));
     if (tma_supported(nm_))
-      for (int q = 0; q < 7; ++q) PMGB_RET(make_spec_tensor_maps<T>(nm_, B_, spec_[q], &tmy_[q], &tmz_[q], &tmf_[q], &tma_[q]));
+      for (int q = 0; q < 7; ++q) PMGB_RET(make_spec_tensor_maps<T>(nm_, B_, spec_[q], &tmy_[q], &tmz_[q], &tmf_[q]));
     PMGB_CK(cudaMemcpyAsync(omega_, omega, sizeof(T) * B_ * N_, cudaMemcpyDeviceToDevice, st_));
     PMGB_RET(tables(theta));
     return PM_OK;
@@ -1380,8 +1380,8 @@ class Engine : public EngineBase {
       za.out[1] = nullptr;
       prof_.begin(st_, P_Z_ADJ, use_tma_ ? 2 : 1);
       if (use_tma_) {
-        const CUtensorMap pm2[2] = {tma_[4], tma_[5]};
-        PMGB_RET(fft_fused_tma<T>(nm_, true, pm2, &tma_[0], za, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));   // psi -> spec_[0]
+        const CUtensorMap pm2[2] = {tmf_[4], tmf_[5]};
+        PMGB_RET(fft_fused_tma<T>(nm_, true, pm2, &tmf_[0], za, tw_, WaitCtl{dev_err_, first_wait_}, nsm_, st_));   // psi -> spec_[0]
         PMGB_RET(fft_fused_z<T>(nm_, za, true, false, tw_, st_));
       } else {
         PMGB_RET(fft_fused_z<T>(nm_, za, true, true, tw_, st_));
@@ -1678,7 +1678,7 @@ class Engine : public EngineBase {
   int* err_host_ = nullptr;   // set by a bounded device wait that gave up (host memory)
   int* dev_err_ = nullptr;    // its device address
   int first_wait_ = -1;   // spin limit of the TMA passes' first wait (test hook)
-  CUtensorMap tmy_[7], tmz_[7], tmf_[7], tma_[7];   // y, z and fused z passes (force, adjoint) of spec_[q]
+  CUtensorMap tmy_[7], tmz_[7], tmf_[7];   // y, z and fused z passes of spec_[q]
 };
 
 template <typename T>

@@ -97,10 +97,9 @@ template <typename T>
 int fft_ymerge_tma(int n, int batch, const CUtensorMap* pmaps, cx_t<T>* p1, const cx_t<T>* tw, const WaitCtl& wc, int nsm,
                    cudaStream_t st);
 // tensor maps of one spectrum buffer for the y pass (box along y), the z pass (box along z) and
-// the fused z passes of the force and of the adjoint (boxes along z of their tiles' columns)
+// the fused z passes (box along z of their tile's columns)
 template <typename T>
-int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap,
-                          CUtensorMap* amap);
+int make_spec_tensor_maps(int n, int batch, cx_t<T>* buf, CUtensorMap* ymap, CUtensorMap* zmap, CUtensorMap* fmap);
 
 // Set the dynamic shared-memory limit of a kernel once per device.
 void ensure_smem_attr(const void* fn, int bytes);
