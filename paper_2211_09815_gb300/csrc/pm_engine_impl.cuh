@@ -1106,7 +1106,7 @@ class Engine : public EngineBase {
       return PM_OK;
     };
     static const int kTiles[][3] = {{3, 4, 4}, {3, 3, 5}, {3, 3, 4}, {2, 4, 5}, {2, 4, 4}, {3, 3, 3},
-                                    {2, 3, 5}, {4, 4, 4}, {3, 4, 5}, {3, 5, 4}};
+                                    {2, 3, 5}, {4, 4, 4}, {3, 4, 5}, {3, 5, 4}, {2, 3, 6}, {2, 2, 6}, {2, 2, 7}};
     const int lg = ilog2(nm_);
     const long long sis = 2 * spec_len_cx(nm_);
     pm_tuning best = tune_;
