@@ -481,12 +481,13 @@ class Engine : public EngineBase {
 
   int op_fft(int dir, const void* in, void* out) override {
     have_fwd_ = false;
-    const long long tot = (long long)B_ * nm_ * nm_ * (nm_ / 2 + 1);
+    const long long rows = (long long)B_ * nm_ * nm_;
+    const int grid = (int)std::min<long long>((rows + 7) / 8, 8LL * nsm_);
     if (dir < 0) {
       PMGB_RET(r2c_real(nm_, (const T*)in, (long long)M_, spec_[0]));
-      k_spec_to_std<T><<<1024, 256, 0, st_>>>(spec_[0], (C*)out, nm_, tot);
+      k_spec_std<T, true><<<grid, 256, 0, st_>>>(spec_[0], (C*)out, nm_, rows);
     } else {
-      k_std_to_spec<T><<<1024, 256, 0, st_>>>((const C*)in, spec_[0], nm_, tot);
+      k_spec_std<T, false><<<grid, 256, 0, st_>>>((const C*)in, spec_[0], nm_, rows);
       PMGB_CK(cudaGetLastError());
       PMGB_RET(c2r_real(nm_, spec_[0], (T*)out, (long long)M_));
     }

@@ -1416,32 +1416,23 @@ k_power_grad(cx_t<T>* spec, PowerRuns pr, long long is, int nb, const double* __
   }
 }
 
-// numpy rfftn layout <-> main + side spectrum layout (for the FFT operator entry point)
-template <typename T>
-__global__ void k_spec_to_std(const cx_t<T>* __restrict__ spec, cx_t<T>* __restrict__ out, int n, long long total) {
-  const int h = n / 2 + 1;
-  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < total; u += (long long)gridDim.x * blockDim.x) {
-    const long long per = (long long)n * n * h;
-    const long long b = u / per, r = u % per;
-    const int k = (int)(r % h);
-    const long long row = r / h;
-    const cx_t<T>* base = spec + b * spec_len_cx(n);
-    const long long mrow = spec_row(n, spec_lzb(n), (int)(row / n), (int)(row % n));
-    out[u] = k < n / 2 ? base[mrow * (n / 2) + k] : base[spec_main_len(n) + row];
-  }
-}
-template <typename T>
-__global__ void k_std_to_spec(const cx_t<T>* __restrict__ in, cx_t<T>* __restrict__ spec, int n, long long total) {
-  const int h = n / 2 + 1;
-  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < total; u += (long long)gridDim.x * blockDim.x) {
-    const long long per = (long long)n * n * h;
-    const long long b = u / per, r = u % per;
-    const int k = (int)(r % h);
-    const long long row = r / h;
-    cx_t<T>* base = spec + b * spec_len_cx(n);
-    const long long mrow = spec_row(n, spec_lzb(n), (int)(row / n), (int)(row % n));
-    if (k < n / 2) base[mrow * (n / 2) + k] = in[u];
-    else base[spec_main_len(n) + row] = in[u];
+// numpy rfftn layout <-> main + side spectrum layout (for the FFT operator entry point), a warp per
+// row of the mesh: the odd row length n/2 + 1 of the numpy layout then needs no division.
+template <typename T, bool TO_STD>
+__global__ void __launch_bounds__(256)
+k_spec_std(const cx_t<T>* __restrict__ in, cx_t<T>* __restrict__ out, int n, long long rows) {
+  using C = cx_t<T>;
+  const int lgn = 31 - __clz(n), half = n / 2, lane = threadIdx.x & 31;
+  for (long long row = blockIdx.x * 8LL + (threadIdx.x >> 5); row < rows; row += gridDim.x * 8LL) {
+    const long long b = row >> (2 * lgn), r = row & ((1LL << (2 * lgn)) - 1);
+    const long long main = b * spec_len_cx(n) + spec_row(n, spec_lzb(n), (int)(r >> lgn), (int)r & (n - 1)) * half;
+    const long long side = b * spec_len_cx(n) + spec_main_len(n) + r, std = row * (half + 1);
+    const C* src = in + (TO_STD ? main : std);
+    C* dst = out + (TO_STD ? std : main);
+    const C last = lane == 0 ? in[TO_STD ? side : std + half] : cmake<C>(0, 0);
+#pragma unroll 8
+    for (int k = lane; k < half; k += 32) dst[k] = src[k];
+    if (lane == 0) out[TO_STD ? std + half : side] = last;
   }
 }
 
