@@ -1586,13 +1586,13 @@ class Engine : public EngineBase {
   int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1, Gi_ = 1;   // grids of the particle loops
 
   // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
-  // resident on all SMs, of a batch of small instances fewer, up to 16 particles to a thread.
-  // (Several whole waves scatter the blocks in flight over the lattice as they drift apart:
-  // adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3 and 1024^3, with one 102, 742
-  // and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470 with one.  The sums at the
-  // end of an adjoint block cost as much as several particles: 8 x 64^3 particles 177 us with one
-  // to a thread, 91 with 27.  But one wave over 16 instances of 128^3 mixes their meshes in the L2:
-  // 1204 us against 836 with one wave for each.)
+  // resident on all SMs, for each instance, or where an instance is no more than kMaxRedBlocks
+  // blocks of particles, for the batch.  (Several whole waves scatter the blocks in flight over the
+  // lattice as they drift apart: adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3
+  // and 1024^3, with one 102, 742 and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470
+  // with one.  The sums at the end of an adjoint block cost as much as several particles: 8 x 64^3
+  // particles 177 us with one to a thread, 91 with 27 in one wave, 106 in one and a half.  But one
+  // wave over 16 instances of 128^3 mixes their meshes in the L2: 1204 us against 836 with one each.)
   int wave_grid(const void* fn, long long work) const {
     const long long need = (work + kPtclThreads - 1) / kPtclThreads;
     int occ = 0;
@@ -1600,8 +1600,9 @@ class Engine : public EngineBase {
       (void)cudaGetLastError();
       occ = 1;
     }
-    const long long wave = std::min<long long>((long long)occ * nsm_, kMaxRedBlocks);
-    return (int)std::max<long long>(1, std::min(need, std::min(wave, std::max(wave / B_, need / 16))));
+    long long blocks = std::min<long long>((long long)occ * nsm_, kMaxRedBlocks);
+    if (need <= kMaxRedBlocks) blocks /= B_;
+    return (int)std::max<long long>(1, std::min(need, blocks));
   }
   long long N_ = 0, M_ = 0, bytes_ = 0;
   T mass_ = 1, inv_kfp_ = 1;
