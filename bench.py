@@ -507,35 +507,29 @@ def run_ours(args, rank, world, local_rank):
 
 
 def run_op_case(args):
-    """The force and force-VJP operators at the final state of a full forward run of the
-    chosen workload (late-time clustering), for ncu captures: a warm-up pair, then one pair
-    between cudaProfilerStart/Stop (one forward and one adjoint force chain)."""
+    """One gradient evaluation of a single step, a = 0.9 -> 1, from the Zel'dovich state at
+    a = 0.9 (late-time displacements) at the chosen workload's size, for ncu captures: a
+    warm-up evaluation, then one between cudaProfilerStart/Stop (two forward and two adjoint
+    force chains with the gathers, kicks and drifts of a simulation step)."""
     import torch
     from paper_2211_09815_gb300 import build, inputs, pm
     build.build()
-    box, nm, npc, n = WORKLOADS[args.workload]
-    N = npc ** 3
+    box, nm, npc, _ = WORKLOADS[args.workload]
     om = torch.from_numpy(inputs.white_noise(npc, 1)).to("cuda")
-    ctx = pm.PMContext(box, nm, npc, n, [THETA], om)
-    # the deposit and x pass as separate kernels, the form the autotuner picks at 1024^3
-    ctx.set_tuning({"fused_x": args.fused_x})
-    disp = torch.empty(3 * N, device="cuda")
-    ctx.forward(disp=disp)
-    pi = torch.ones(3 * N, device="cuda") * 1e-3
-    acc = torch.empty(3 * N, device="cuda")
-    alpha = torch.empty(3 * N, device="cuda")
-    ctx.op_force(disp, acc)
-    ctx.op_force_vjp(disp, pi, acc, alpha)
+    ctx = pm.PMContext(box, nm, npc, 1, [THETA], om, a0=0.9)
+    if args.fused_x:
+        ctx.set_tuning({"fused_x": args.fused_x})
+    target = torch.zeros(nm ** 3, device="cuda")
+    gw = torch.empty(npc ** 3, device="cuda")
+    ctx.gradient(target, grad_omega=gw)
     torch.cuda.synchronize()
-    # the second pair is bracketed for `ncu --profile-from-start off`
+    # the second evaluation is bracketed for `ncu --profile-from-start off`
     torch.cuda.profiler.start()
-    ctx.op_force(disp, acc)
-    ctx.op_force_vjp(disp, pi, acc, alpha)
+    ctx.gradient(target, grad_omega=gw)
     torch.cuda.synchronize()
     torch.cuda.profiler.stop()
     ctx.close()
-    print(json.dumps({"op_case": args.workload, "acc_rms": float(acc.pow(2).mean().sqrt()),
-                      "alpha_rms": float(alpha.pow(2).mean().sqrt())}))
+    print(json.dumps({"op_case": args.workload, "grad_rms": float(gw.pow(2).mean().sqrt())}))
 
 
 def run_fft_compare(args):
@@ -847,7 +841,7 @@ def run_precision_study(args):
 
 
 TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "ncu_traffic_medium_force_chains.md")
-TRAFFIC_NOTE = ("ncu DRAM read + write bytes of every kernel of one forward and one adjoint force chain at "
+TRAFFIC_NOTE = ("ncu DRAM read + write bytes of every kernel of one forward and one adjoint step at "
                 "256^3/512^3, scaled x8 to 512^3/1024^3 (profiles/ncu_traffic_medium_force_chains.md)")
 
 
@@ -902,7 +896,7 @@ def main():
     ap.add_argument("--oracle-steps", type=int, default=2, help="steps of the 128^3 case of --oracle-full")
     ap.add_argument("--fused-x", type=int, default=0, help="--op-case: pm_tuning.fused_x (0: separate passes)")
     ap.add_argument("--op-case", action="store_true",
-                    help="run one force and one force-VJP operator call (no timing), for profilers")
+                    help="run one single-step gradient evaluation (no timing), for profilers")
     args = ap.parse_args()
     rank = int(os.environ.get("RANK", 0))
     world = int(os.environ.get("WORLD_SIZE", 1))
