@@ -155,11 +155,12 @@ class Engine : public EngineBase {
       PMGB_CK(cudaGetDevice(&dev));
       PMGB_CK(cudaDeviceGetAttribute(&nsm_, cudaDevAttrMultiProcessorCount, dev));
     }
-    // particle loops: whole waves of resident blocks (grid-stride loops, every thread the
-    // same share), so that no partial last wave leaves SMs idle; G_ is also the number of
-    // per-block partial sums of the reductions
+    // particle loops (grid-stride): wave_grid; G_ is also the number of per-block partial sums of
+    // the adjoint gather, Go_ of the other reductions over particles, whose kernels need few
+    // registers and take more blocks (k_adjoint_init at 128^3 particles: 304 blocks 52 us, 1024 36)
     hf_ = cfg->half_force != 0 && sizeof(T) == 4;
     G_ = wave_grid((const void*)gather_adj_fn(), N_);
+    Go_ = (int)std::min<long long>((N_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks);
     Gf_ = wave_grid((const void*)gather_fwd_fn(), N_);
     // The operators' gathers need few registers.  At 1024^3 (a 17 GB force mesh) more than two
     // blocks per SM in flight span more pages than the address translation holds: force 28.9 ->
@@ -319,9 +320,9 @@ class Engine : public EngineBase {
     PMGB_CK(cudaMemsetAsync(pimax_, 0, sizeof(unsigned) * 3 * B_, st_));
     const int nobs = n_ + 1 + (int)interp_.size();   // theta-term slots of the observations
     const bool obs_theta = snap_gmom_ || (!interp_.empty() && (interp_gdisp_ || interp_gdens_));
-    if (obs_theta) PMGB_CK(cudaMemsetAsync(obs_part_, 0, sizeof(double) * nobs * B_ * G_, st_));
+    if (obs_theta) PMGB_CK(cudaMemsetAsync(obs_part_, 0, sizeof(double) * nobs * B_ * Go_, st_));
     prof_.begin(st_, P_OTHER, 1);
-    k_adjoint_init<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, mass_, s_, (const T*)djdd, (const T*)djdx,
+    k_adjoint_init<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(geo_, mass_, s_, (const T*)djdd, (const T*)djdx,
                                                               (const T*)djdp, xi_, pi_, pimax_);
     prof_.end(st_, P_OTHER);
     PMGB_CK(cudaGetLastError());
@@ -331,7 +332,7 @@ class Engine : public EngineBase {
       const int q = snap_of(j);
       if (q >= 0 && (snap_gdisp_ || snap_gdens_)) {
         prof_.begin(st_, P_OTHER, 1);
-        k_obs_cotangent<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(
+        k_obs_cotangent<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(
             geo_, mass_, s_, snap_gdens_ ? snap_gdens_ + (long long)q * B_ * M_ : nullptr,
             snap_gdisp_ ? snap_gdisp_ + (long long)q * B_ * 3 * N_ : nullptr, xi_);
         prof_.end(st_, P_OTHER);
@@ -341,11 +342,11 @@ class Engine : public EngineBase {
       for (size_t k = 0; k < interp_.size(); ++k)
         if (interp_[k].j == j && (interp_gdisp_ || interp_gdens_)) {
           prof_.begin(st_, P_OTHER, 1);
-          k_obs_interp<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(
+          k_obs_interp<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(
               geo_, mass_, s_, p_, obs_fac_ + (long long)k * B_,
               interp_gdens_ ? interp_gdens_ + (long long)k * B_ * M_ : nullptr,
               interp_gdisp_ ? interp_gdisp_ + (long long)k * B_ * 3 * N_ : nullptr, xi_, pi_,
-              obs_part_ + (long long)(n_ + 1 + k) * B_ * G_, pimax_);
+              obs_part_ + (long long)(n_ + 1 + k) * B_ * Go_, pimax_);
           prof_.end(st_, P_OTHER);
           PMGB_CK(cudaGetLastError());
         }
@@ -354,7 +355,7 @@ class Engine : public EngineBase {
       const T* vmom = (q >= 0 && snap_gmom_) ? snap_gmom_ + (long long)q * B_ * 3 * N_ : nullptr;
       if (vmom) {
         prof_.begin(st_, P_OTHER, 1);
-        k_obs_momentum<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, pi_, vmom, obs_c_, j, n_ + 1, 0, nullptr,
+        k_obs_momentum<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(geo_, pi_, vmom, obs_c_, j, n_ + 1, 0, nullptr,
                                                                   nullptr, pimax_);
         prof_.end(st_, P_OTHER);
         PMGB_CK(cudaGetLastError());
@@ -381,8 +382,8 @@ class Engine : public EngineBase {
       PMGB_CK(cudaGetLastError());
       if (vmom) {
         prof_.begin(st_, P_OTHER, 1);
-        k_obs_momentum<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, pi_, vmom, obs_c_, j, n_ + 1, 1, a_,
-                                                                  obs_part_ + (long long)j * B_ * G_, pimax_);
+        k_obs_momentum<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(geo_, pi_, vmom, obs_c_, j, n_ + 1, 1, a_,
+                                                                  obs_part_ + (long long)j * B_ * Go_, pimax_);
         prof_.end(st_, P_OTHER);
         PMGB_CK(cudaGetLastError());
       }
@@ -412,7 +413,7 @@ class Engine : public EngineBase {
     in.step_stride = 2 * B_;
     k_final_theta<<<(B_ + 31) / 32, 32, 0, st_>>>(in, theta_out_);
     if (obs_theta) {
-      k_sum_partials<<<nobs * B_, 256, 0, st_>>>(obs_part_, G_, obs_sums_, 1.0);
+      k_sum_partials<<<nobs * B_, 256, 0, st_>>>(obs_part_, Go_, obs_sums_, 1.0);
       k_obs_theta<<<(B_ + 31) / 32, 32, 0, st_>>>(obs_sums_, obs_w_, nobs, B_, theta_out_);
     }
     prof_.end(st_, P_OTHER);
@@ -726,7 +727,7 @@ class Engine : public EngineBase {
     if (interp_dens_) {
       unsigned long long* acc = reinterpret_cast<unsigned long long*>(fvec_);
       PMGB_CK(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * B_ * M_, st_));
-      k_scatter<T, 1><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(geo_, out, nullptr, acc, e_d_, nullptr);
+      k_scatter<T, 1><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(geo_, out, nullptr, acc, e_d_, nullptr);
       k_density_out<T><<<1024, 256, 0, st_>>>((const long long*)acc, interp_dens_ + (long long)k * B_ * M_,
                                               (long long)B_ * M_, (T)(mass_ * std::ldexp(1.0, -e_d_)));
       PMGB_CK(cudaGetLastError());
@@ -856,7 +857,7 @@ class Engine : public EngineBase {
     PMGB_RET(upload_grow(&obs_w_, ow, obs_w_n_));
     if (obs_sums_n_ < (long long)(n1 + nq) * B_) {
       PMGB_RET(alloc(&obs_sums_, (long long)(n1 + nq) * B_));
-      PMGB_RET(alloc(&obs_part_, (long long)(n1 + nq) * B_ * G_));
+      PMGB_RET(alloc(&obs_part_, (long long)(n1 + nq) * B_ * Go_));
       obs_sums_n_ = (long long)(n1 + nq) * B_;
     }
     PMGB_RET(upload(&wpa_, wpa));
@@ -1487,10 +1488,10 @@ class Engine : public EngineBase {
   // transpose adds its part.  Leaves Omega^ in spec_[0].  27 launches.
   int lpt2_adjoint() {
     const long long lis = spec_len_cx(np_);
-    k_ic_adj_prep<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(xi_, pi_, s2_, N_, d2_, gd2_, rmesh(1), rmesh(2),
-                                                             rmesh(3), 2 * lis, part_, part_ + (long long)B_ * G_);
+    k_ic_adj_prep<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(xi_, pi_, s2_, N_, d2_, gd2_, rmesh(1), rmesh(2),
+                                                             rmesh(3), 2 * lis, part_, part_ + (long long)B_ * Go_);
     PMGB_CK(cudaGetLastError());
-    k_sum_partials<<<2 * B_, 256, 0, st_>>>(part_, G_, scal_ + 9 * B_, 1.0);
+    k_sum_partials<<<2 * B_, 256, 0, st_>>>(part_, Go_, scal_ + 9 * B_, 1.0);
     PMGB_CK(cudaGetLastError());
     RowJob<T> job{};
     for (int c = 0; c < 3; ++c) job.b[c] = RowBuf<T>{rmesh(1 + c), 2 * lis, spec_[1 + c]};
@@ -1550,10 +1551,10 @@ class Engine : public EngineBase {
   int ic_adjoint(void* djdw) {
     const long long lis = spec_len_cx(np_);
     if (lpt2_) PMGB_RET(lpt2_adjoint());
-    k_ic_adj_prep<T><<<dim3(G_, B_), kPtclThreads, 0, st_>>>(xi_, pi_, s1_, N_, d1_, gd_, rmesh(1), rmesh(2),
-                                                             rmesh(3), 2 * lis, part_, part_ + (long long)B_ * G_);
+    k_ic_adj_prep<T><<<dim3(Go_, B_), kPtclThreads, 0, st_>>>(xi_, pi_, s1_, N_, d1_, gd_, rmesh(1), rmesh(2),
+                                                             rmesh(3), 2 * lis, part_, part_ + (long long)B_ * Go_);
     PMGB_CK(cudaGetLastError());
-    k_sum_partials<<<2 * B_, 256, 0, st_>>>(part_, G_, scal_ + 2 * B_, 1.0);
+    k_sum_partials<<<2 * B_, 256, 0, st_>>>(part_, Go_, scal_ + 2 * B_, 1.0);
     PMGB_CK(cudaGetLastError());
     // 3 R2C of sbar (in place: real input in the same buffer) and the R2C of omega
     RowJob<T> job{};
@@ -1582,7 +1583,7 @@ class Engine : public EngineBase {
 
   pm_config cfg_{};
   cudaStream_t st_ = 0;
-  int B_ = 1, np_ = 0, nm_ = 0, n_ = 0, lgN_ = 0, e_d_ = 0, G_ = 1, Gm_ = 1, Gz_ = 1, nck_ = 0, maxn2_ = 0;
+  int B_ = 1, np_ = 0, nm_ = 0, n_ = 0, lgN_ = 0, e_d_ = 0, G_ = 1, Go_ = 1, Gm_ = 1, Gz_ = 1, nck_ = 0, maxn2_ = 0;
   int Gf_ = 1, Gc_ = 1, Gb1_ = 1, Gb4_ = 1, Gof_ = 1, Goa_ = 1, Gpm_ = 1, Gi_ = 1;   // grids of the particle loops
 
   // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
