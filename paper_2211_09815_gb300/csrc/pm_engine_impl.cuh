@@ -159,7 +159,7 @@ class Engine : public EngineBase {
     // the adjoint gather, Go_ of the other reductions over particles, whose kernels need few
     // registers and take more blocks (k_adjoint_init at 128^3 particles: 304 blocks 52 us, 1024 36)
     hf_ = cfg->half_force != 0 && sizeof(T) == 4;
-    G_ = wave_grid((const void*)gather_adj_fn(), N_);
+    G_ = wave_grid((const void*)gather_adj_fn(), N_, true);
     Go_ = (int)std::min<long long>((N_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks);
     Gf_ = wave_grid((const void*)gather_fwd_fn(), N_);
     // The operators' gathers need few registers.  At 1024^3 (a 17 GB force mesh) more than two
@@ -1588,13 +1588,13 @@ class Engine : public EngineBase {
 
   // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
   // resident on all SMs, for each instance, or where an instance is no more than kMaxRedBlocks
-  // blocks of particles, for the batch.  (Several whole waves scatter the blocks in flight over the
+  // blocks of particles, for the batch; with `sums` always for each instance, so that sums of
+  // doubles are grouped alike in a batch and alone, and their bits the same.  (Several whole waves scatter the blocks in flight over the
   // lattice as they drift apart: adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3
   // and 1024^3, with one 102, 742 and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470
-  // with one.  The sums at the end of an adjoint block cost as much as several particles: 8 x 64^3
-  // particles 177 us with one to a thread, 91 with 27 in one wave, 106 in one and a half.  But one
-  // wave over 16 instances of 128^3 mixes their meshes in the L2: 1204 us against 836 with one each.)
-  int wave_grid(const void* fn, long long work) const {
+  // with one.  One wave over 16 instances of 128^3 mixes their meshes in the L2: adjoint gather
+  // 1204 us against 836 with one each.)
+  int wave_grid(const void* fn, long long work, bool sums = false) const {
     const long long need = (work + kPtclThreads - 1) / kPtclThreads;
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kPtclThreads, 0) != cudaSuccess || occ < 1) {
@@ -1602,7 +1602,7 @@ class Engine : public EngineBase {
       occ = 1;
     }
     long long blocks = std::min<long long>((long long)occ * nsm_, kMaxRedBlocks);
-    if (need <= kMaxRedBlocks) blocks /= B_;
+    if (!sums && need <= kMaxRedBlocks) blocks /= B_;
     return (int)std::max<long long>(1, std::min(need, blocks));
   }
   long long N_ = 0, M_ = 0, bytes_ = 0;
