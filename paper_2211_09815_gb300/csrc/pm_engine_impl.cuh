@@ -982,9 +982,9 @@ class Engine : public EngineBase {
     return PM_OK;
   }
 
-  // Bins of the tile-owner deposit, sized for the smallest tile the tuner may choose
-  // (2^9 cells); the tile shape and threads per tile of the density-only deposit (forward)
-  // and of the density + pi deposit (adjoint) are set separately (pm_tuning).
+  // Bins of the tile-owner deposit, sized for every tile shape that may run (max_bin_keys);
+  // the tile shape and threads per tile of the density-only deposit (forward) and of the
+  // density + pi deposit (adjoint) are set separately (pm_tuning).
   int bin_setup() {
     // Deposit shapes.  Tiles long in x: the lattice neighbours of a warp spread over more rows'
     // lines, and the write-out stores whole ones.  2^12 cells for the density, 2^11 with the pi sums
@@ -1000,16 +1000,15 @@ class Engine : public EngineBase {
     tune_.tma_columns = 1;
     // (the density deposit of 128^3 meshes alone is faster fused: 145 against 147 us a force)
     tune_.fused_x = nm_ == 128 && !cfg_.fixed_state ? 1 : 0;
-    const BinGeo smallest = make_bin_geo(ilog2(nm_), 3, 3, 3);
-    const long long maxbin = (long long)B_ * smallest.nkeys + 1;
+    max_bins_ = (long long)B_ * max_bin_keys(ilog2(nm_)) + 1;
     PMGB_RET(alloc(&bkeys_, (long long)B_ * N_));
     PMGB_RET(alloc(&brec0_, (long long)B_ * N_));
     PMGB_RET(alloc(&brec1_, (long long)B_ * N_));
-    PMGB_RET(alloc(&bcount_, maxbin));
-    PMGB_RET(alloc(&bstart_, maxbin));
-    PMGB_RET(alloc(&bcursor_, maxbin));
-    PMGB_RET(alloc(&bsums_, (maxbin + kScanBlock - 1) / kScanBlock));
-    PMGB_CK(cudaMemsetAsync(bcount_, 0, sizeof(unsigned) * maxbin, st_));
+    PMGB_RET(alloc(&bcount_, max_bins_));
+    PMGB_RET(alloc(&bstart_, max_bins_));
+    PMGB_RET(alloc(&bcursor_, max_bins_));
+    PMGB_RET(alloc(&bsums_, (max_bins_ + kScanBlock - 1) / kScanBlock));
+    PMGB_CK(cudaMemsetAsync(bcount_, 0, sizeof(unsigned) * max_bins_, st_));
     ensure_smem_attr((const void*)k_pull_scatter<T, 4, 256>, 4 * 8 * 2048);
     ensure_smem_attr((const void*)k_pull_scatter<T, 4, 512>, 4 * 8 * 2048);
     apply_tuning();
@@ -1033,12 +1032,6 @@ class Engine : public EngineBase {
       bgf1_ = geo(fused_rows<T>(nm_, 1));
       bgf4_ = geo(fused_rows<T>(nm_, 4));
     }
-  }
-  // tile extents: x at least 4 cells (vector write-out), 2^9..2^maxl cells (shared memory:
-  // 2^12 cells x 8 B for the density alone, 2^11 x 32 B with the pi sums)
-  static bool tile_ok(const int* l, int maxl) {
-    return l[0] >= 0 && l[1] >= 0 && l[2] >= 2 && l[0] + l[1] + l[2] >= 9 && l[0] + l[1] + l[2] <= maxl &&
-           l[0] <= 10 && l[1] <= 10 && l[2] <= 10;
   }
   int get_tuning(pm_tuning* t) override {
     *t = tune_;
@@ -1275,6 +1268,7 @@ class Engine : public EngineBase {
   int deposit(const T* s, const T* pi, T* dout, long long dis, const BinGeo& bg, int nt, bool precounted = false,
               const FusedOut<T>* fo = nullptr, const SepTargets* tg = nullptr) {
     const long long nbin = (long long)B_ * bg.nkeys + 1;
+    if (nbin > max_bins_) return PM_ERR_STATE;
     const int nscan = (int)((nbin + kScanBlock - 1) / kScanBlock);
     if (!precounted) k_bin_count<T><<<dim3(Gc_, B_), kPtclThreads, 0, st_>>>(geo_, bg, s, bcount_, bkeys_);
     k_scan_blocks<<<nscan, 256, 0, st_>>>(bcount_, bstart_, bsums_, nbin);
@@ -1640,6 +1634,7 @@ class Engine : public EngineBase {
   pm_tuning tune_{};
   bool tuned_ = false;           // pm_set_tuning was called
   long long* sacc_ = nullptr;    // integer mesh of the small deposits, zero between calls
+  long long max_bins_ = 0;       // length of bcount_, bstart_ and bcursor_
   unsigned *bkeys_ = nullptr, *bcount_ = nullptr, *bstart_ = nullptr, *bcursor_ = nullptr, *bsums_ = nullptr;
   V4<T> *brec0_ = nullptr, *brec1_ = nullptr;
   C* spec_[7] = {};

@@ -14,6 +14,7 @@
 //  k_lpt_hess, k_lpt_source, k_lpt_source_adj, k_lpt_hess_adj, k_ic_state2
 #pragma once
 #include <cuda_fp16.h>
+#include "bin_geo.h"
 #include "common.cuh"
 #include "pm_internal.h"
 
@@ -276,29 +277,7 @@ template <> inline int fixed_top<float>(int lgN) { return 61 - lgN < 30 ? 61 - l
 template <> inline int fixed_top<double>(int lgN) { return 61 - lgN; }
 
 // ------------------------------------------------------------------ deposit bins
-// Bins of the tile-owner deposit (bin_kernels.cuh): mesh tiles of 2^lx x 2^ly x 2^lz cells
-// (x = array axis 2), and per tile a class of three bits, set when the particle's cell is on
-// the tile's last layer along x, y or z (its CIC cloud reaches into the next tile there).
-struct BinGeo {
-  int lx, ly, lz;       // log2 of the tile extent along axes 2, 1, 0
-  int ntx, nty, ntz;    // tiles per axis
-  int ntiles;           // per instance
-  long long nkeys;      // bins per instance = 8 ntiles
-};
-
-inline BinGeo make_bin_geo(int lg_nm, int lx, int ly, int lz) {
-  BinGeo b;
-  b.lx = lx < lg_nm ? lx : lg_nm;
-  b.ly = ly < lg_nm ? ly : lg_nm;
-  b.lz = lz < lg_nm ? lz : lg_nm;
-  b.ntx = 1 << (lg_nm - b.lx);
-  b.nty = 1 << (lg_nm - b.ly);
-  b.ntz = 1 << (lg_nm - b.lz);
-  b.ntiles = b.ntx * b.nty * b.ntz;
-  b.nkeys = 8LL * b.ntiles;
-  return b;
-}
-
+// (tiles and bins: bin_geo.h)
 // class bits of a cell: on the last layer of its tile along x (bit 0), y (bit 1), z (bit 2)
 __device__ __forceinline__ unsigned bin_class(const BinGeo& bg, const int c[3]) {
   const unsigned mx = (1u << bg.lx) - 1, my = (1u << bg.ly) - 1, mz = (1u << bg.lz) - 1;
