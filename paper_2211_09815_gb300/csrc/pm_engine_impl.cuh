@@ -438,15 +438,15 @@ class Engine : public EngineBase {
   }
 
   // The operators read the caller's particles where they lie: the deposit reads all of them
-  // before the gather writes a result.  Only inputs that overlap an output are copied first
-  // (into buf).
+  // before the gather writes a result.  Only inputs that overlap an output, or that lie off
+  // their elements' alignment, which kernels cannot read, are copied first (into buf).
   int op_input(const void* in, const void* out0, long long n0, const void* out1, long long n1, T* buf, const T** use) {
     auto meets = [&](const void* out, long long n) {
       const uintptr_t a = (uintptr_t)in, b = (uintptr_t)out;
       return out && a < b + sizeof(T) * n && b < a + sizeof(T) * B_ * 3 * N_;
     };
     *use = (const T*)in;
-    if (meets(out0, n0) || meets(out1, n1)) {
+    if (meets(out0, n0) || meets(out1, n1) || (uintptr_t)in % sizeof(T)) {
       PMGB_CK(cudaMemcpyAsync(buf, in, sizeof(T) * B_ * 3 * N_, cudaMemcpyDeviceToDevice, st_));
       *use = buf;
     }
