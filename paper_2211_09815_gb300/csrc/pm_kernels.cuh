@@ -1210,21 +1210,22 @@ k_power_max(const cx_t<T>* __restrict__ spec, PowerRuns pr, long long is, int nb
     if (bin >= nb) continue;                             // |n| only grows along the run
     cx_t<T> v[8];
     load_run(p, pr.lglen, v);
-    float m = 0.f;
+    // the powers are non-negative: their bit patterns order like the values, NaN above infinity
+    // (its sign cleared), so that a NaN stays the maximum
+    unsigned m = 0u;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       if (k >= (1 << pr.lglen)) break;
       const int n2 = n01 + (kx + k) * (kx + k);
       if (n2 >= (bin + 1) * (bin + 1)) {
-        atomicMax(&smax[bin], __float_as_uint(m));
-        m = 0.f;
+        atomicMax(&smax[bin], m);
+        m = 0u;
         while (n2 >= (bin + 1) * (bin + 1)) ++bin;
         if (bin >= nb) break;
       }
-      const float q = power_up(v[k], kx + k == 0 ? 0 : 1);
-      m = q == q ? fmaxf(m, q) : q;
+      m = max(m, __float_as_uint(power_up(v[k], kx + k == 0 ? 0 : 1)) & 0x7FFFFFFFu);
     }
-    if (bin < nb) atomicMax(&smax[bin], __float_as_uint(m));
+    if (bin < nb) atomicMax(&smax[bin], m);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < nb; i += kPowerThreads)
