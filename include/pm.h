@@ -256,6 +256,10 @@ long long pm_scratch_bytes(const pm_ctx* ctx);
  *                          deposit and x pass of the R2C in one kernel, meshes 128..1024);
  *                          clear = it writes real meshes and a separate x pass transforms
  *                          them (the tile shapes above apply to that form)
+ * Deposits of few particles (nq batch n_ptcl^3 <= 2^18 and nq batch n_mesh^3 <= 2^21, nq = 1
+ * for the density and 4 with the pi sums) need no tiles: there the default shape (tile and
+ * threads, not fused) stands for a deposit by global atomics, with the same sums, which is
+ * what such a context runs until another shape is set for that deposit.
  */
 typedef struct pm_tuning {
   int tile_log2_density[3];
@@ -277,7 +281,8 @@ int pm_set_tuning(pm_ctx* ctx, const pm_tuning* t);
 
 /*
  * Autotuner: times every candidate deposit tile shape x threads per tile (for the forward
- * and the adjoint deposit separately), then each deposit fused with the x pass against the
+ * and the adjoint deposit separately; in place of the default shape the deposit of few
+ * particles, where that is what runs), then each deposit fused with the x pass against the
  * best separate deposit plus x pass, and both column-pass forms on the context's current
  * particle state (the final state of the last pm_forward, else the Zel'dovich state), each
  * `reps` times with CUDA events on the context's stream (median; reps = 0 means 3), and

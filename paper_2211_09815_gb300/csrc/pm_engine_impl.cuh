@@ -999,7 +999,8 @@ class Engine : public EngineBase {
     tune_.threads_adjoint = 512;
     tune_.tma_columns = 1;
     // (the density deposit of 128^3 meshes alone is faster fused: 145 against 147 us a force)
-    tune_.fused_x = nm_ == 128 && !cfg_.fixed_state ? 1 : 0;
+    tune_.fused_x = nm_ == 128 && !cfg_.fixed_state && !small_rule(1) ? 1 : 0;
+    tune0_ = tune_;
     max_bins_ = (long long)B_ * max_bin_keys(ilog2(nm_)) + 1;
     PMGB_RET(alloc(&bkeys_, (long long)B_ * N_));
     PMGB_RET(alloc(&brec0_, (long long)B_ * N_));
@@ -1048,7 +1049,6 @@ class Engine : public EngineBase {
     if (t->fused_x < 0 || t->fused_x > 3 || (t->fused_x && (fused_rows<T>(nm_, 1) == 0 || cfg_.fixed_state)))
       return PM_ERR_ARG;
     tune_ = *t;
-    tuned_ = true;
     apply_tuning();
     return PM_OK;
   }
@@ -1103,7 +1103,14 @@ class Engine : public EngineBase {
     static const int kTiles[][3] = {{3, 4, 4}, {3, 3, 5}, {3, 3, 4}, {2, 4, 5}, {2, 4, 4}, {3, 3, 3},
                                     {2, 3, 5}, {4, 4, 4}, {3, 4, 5}, {3, 5, 4}, {2, 3, 6}, {2, 2, 6}, {2, 2, 7}};
     const int lg = ilog2(nm_);
-    const long long sis = 2 * spec_len_cx(nm_);
+    // the separate deposit that runs with shapes t
+    auto separate = [&](const pm_tuning& t, int nq, const SepTargets& tg) {
+      const T* pi = nq ? xi_ : nullptr;
+      if (small_deposit(nq != 0, t)) return scatter_small(s_, pi, tg.d, tg.dis, tg);
+      const int* l = nq ? t.tile_log2_adjoint : t.tile_log2_density;
+      return deposit(s_, pi, tg.d, tg.dis, make_bin_geo(lg, l[2], l[1], l[0]),
+                     nq ? t.threads_adjoint : t.threads_density, false, nullptr, &tg);
+    };
     pm_tuning best = tune_;
     double best_ms[3] = {1e30, 1e30, 1e30};
     for (int nq = 0; nq < 2; ++nq) {
@@ -1111,16 +1118,15 @@ class Engine : public EngineBase {
         const int l[3] = {tl[0], tl[1], tl[2]};
         if (!tile_ok(l, nq ? 11 : 12)) continue;
         for (int nt : {256, 512}) {
-          const BinGeo bg = make_bin_geo(lg, l[2], l[1], l[0]);
+          pm_tuning cand = best;
+          std::copy(l, l + 3, nq ? cand.tile_log2_adjoint : cand.tile_log2_density);
+          (nq ? cand.threads_adjoint : cand.threads_density) = nt;
+          cand.fused_x &= nq ? 1 : 2;
           double ms = 0;
-          PMGB_RET(time_it([&]() { return deposit(s_, nq ? xi_ : nullptr, rmesh(0), sis, bg, nt); }, &ms));
+          PMGB_RET(time_it([&]() { return separate(cand, nq, sep_targets(false)); }, &ms));
           if (ms < best_ms[nq]) {
             best_ms[nq] = ms;
-            int* dst = nq ? best.tile_log2_adjoint : best.tile_log2_density;
-            dst[0] = l[0];
-            dst[1] = l[1];
-            dst[2] = l[2];
-            (nq ? best.threads_adjoint : best.threads_density) = nt;
+            best = cand;
           }
         }
       }
@@ -1130,13 +1136,10 @@ class Engine : public EngineBase {
     if (fused_rows<T>(nm_, 1) > 0 && !cfg_.fixed_state) {
       best.fused_x = 0;
       for (int nq = 0; nq < 2; ++nq) {
-        const int* l = nq ? best.tile_log2_adjoint : best.tile_log2_density;
-        const BinGeo bg = make_bin_geo(lg, l[2], l[1], l[0]);
-        const int nt = nq ? best.threads_adjoint : best.threads_density;
         double ms_sep = 0, ms_fused = 0;
         const SepTargets tg = sep_targets(false);
         PMGB_RET(time_it([&]() {
-          PMGB_RET(deposit(s_, nq ? xi_ : nullptr, tg.d, tg.dis, bg, nt, false, nullptr, &tg));
+          PMGB_RET(separate(best, nq, tg));
           RowJob<T> job{};
           job.b[0] = RowBuf<T>{tg.d, tg.dis, spec_[0]};
           if (nq)
@@ -1213,11 +1216,18 @@ class Engine : public EngineBase {
   // in the tile deposit and the sums are exact, so the meshes are the same bit for bit.  The
   // line: the atomics run at about 1e11 per second, 8 nq per particle, against some 20 us that
   // the bins take at least; and the integer mesh is 8 nq bytes per cell, read and cleared.
-  // Shapes set by pm_set_tuning are taken as asked.
   bool small_rule(int nq) const {
     return nq * (long long)B_ * N_ <= (1LL << 18) && nq * (long long)B_ * M_ <= (1LL << 21);
   }
-  bool small_deposit(bool pi) const { return !tuned_ && small_rule(pi ? 4 : 1); }
+  // Within the rule the default shape stands for this deposit (the tuner's candidate of that
+  // shape times it); any other shape, and the fused form, run as asked.
+  bool small_deposit(bool pi) const { return small_deposit(pi, tune_); }
+  bool small_deposit(bool pi, const pm_tuning& t) const {
+    const int* l = pi ? t.tile_log2_adjoint : t.tile_log2_density;
+    const int* l0 = pi ? tune0_.tile_log2_adjoint : tune0_.tile_log2_density;
+    return small_rule(pi ? 4 : 1) && std::equal(l, l + 3, l0) && !(t.fused_x & (pi ? 2 : 1)) &&
+           (pi ? t.threads_adjoint == tune0_.threads_adjoint : t.threads_density == tune0_.threads_density);
+  }
   int scatter_small(const T* s, const T* pi, T* dout, long long dis, const SepTargets& tg) {
     unsigned long long* acc = reinterpret_cast<unsigned long long*>(sacc_);
     const dim3 gp((unsigned)std::min<long long>((N_ + kPtclThreads - 1) / kPtclThreads, kMaxRedBlocks), B_);
@@ -1321,7 +1331,7 @@ class Engine : public EngineBase {
   int force_chain(const T* s, const T* pi, bool keep_density) {
     // delta goes to the real view of spec_[0] (transformed in place) or, when the final
     // density is kept for the objective, to dens_
-    if (!small_deposit(pi != nullptr) && (pi ? fused4_ : fused1_)) {
+    if (pi ? fused4_ : fused1_) {
       // deposit and x pass in one kernel: delta (and pi_c) straight into the half spectra
       FusedOut<T> fo{};
       fo.spec[0] = spec_[0];
@@ -1632,7 +1642,7 @@ class Engine : public EngineBase {
   double fused_ms_[4] = {};   // autotuner: separate and fused deposit times (density, density + pi)   // forward (density) / adjoint (density + pi) deposit fused
   bool counted_ = false;   // the last gather counted the bins of the next deposit
   pm_tuning tune_{};
-  bool tuned_ = false;           // pm_set_tuning was called
+  pm_tuning tune0_{};            // the default shapes
   long long* sacc_ = nullptr;    // integer mesh of the small deposits, zero between calls
   long long max_bins_ = 0;       // length of bcount_, bstart_ and bcursor_
   unsigned *bkeys_ = nullptr, *bcount_ = nullptr, *bstart_ = nullptr, *bcursor_ = nullptr, *bsums_ = nullptr;
