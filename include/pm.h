@@ -239,9 +239,10 @@ const char* pm_last_cuda_error(void);
 long long pm_scratch_bytes(const pm_ctx* ctx);
 
 /*
- * Launch shapes of the tunable passes (not in the paper; they change speed, never
- * results: the CIC sums are exact integers for any tile shape, and the staged and
- * unstaged column passes run the same radix stages).
+ * Launch shapes of the tunable passes (not in the paper; they change speed, not the
+ * results beyond rounding: the CIC sums are exact integers, the same for any tile shape;
+ * staged and unstaged column passes, and fused and separate x passes, run the same radix
+ * stages and may differ in the last bit).
  *   tile_log2_density[3] : log2 of the deposit tile extent along axes (z, y, x), the
  *                          density-only deposit of the forward steps; 9..12 in total,
  *                          x at least 2

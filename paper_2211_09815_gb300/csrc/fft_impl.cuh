@@ -934,7 +934,8 @@ static void launch_c2r4_L(const RowJob<T>& job, int nrows, int dq, void* out, si
                           cudaStream_t st) {
   constexpr bool kRows = sizeof(T) == 4 && has_warp_rows(L);
   if (job.b[3].spec) {
-    // (four components of 128 points: 16 x 256^3 in 1.64 ms as tiles, 1.68 as rows)
+    // (four components of 128 points: 16 x 256^3 in 1.64 ms as tiles, 1.68 as rows; the two forms
+    // round alike, which the reversal of the fixed-point state needs: tests/test_gpu_acc_forms.py)
     if constexpr (kRows && L != 128) launch_rows_c2r4<L, 4>(job, nrows, dq, out, fexp, tw, st);
     else launch_c2r4_LQ<T, L, 4>(job, nrows, dq, out, fexp, tw, st);
   } else {

@@ -998,7 +998,11 @@ class Engine : public EngineBase {
     tune_.threads_density = 256;
     tune_.threads_adjoint = 512;
     tune_.tma_columns = 1;
-    // (the density deposit of 128^3 meshes alone is faster fused: 145 against 147 us a force)
+    // The density deposit of 128^3 meshes is faster fused: force, separate / fused, with 64^3
+    // particles x 2, 4, 8 and 16 instances 162 / 158, 246 / 242, 412 / 405 and 755 / 741 us, 32^3 x 16
+    // 591 / 577, 128^3 x 1 and 4 221 / 205 and 553 / 543 (the VJP's is not: 64^3 x 8 774 / 807; nor are
+    // larger meshes: 128^3 on 256^3 412 / 418, 256^3 on 512^3 2771 / 2861).  In FP64 the two forms are
+    // within 1% of each other at 128^3 to 512^3.  (Few particles: the atomics, see small_deposit.)
     tune_.fused_x = nm_ == 128 && !cfg_.fixed_state && !small_rule(1) ? 1 : 0;
     tune0_ = tune_;
     max_bins_ = (long long)B_ * max_bin_keys(ilog2(nm_)) + 1;
@@ -1058,9 +1062,10 @@ class Engine : public EngineBase {
   // none) and keeps the fastest.  Candidates: deposit tile shapes (2^9..2^11 cells) x 256
   // or 512 threads, separately for the density-only and the density + pi deposit; the
   // y column pass with or without TMA staging.  Each candidate is timed `reps` times with
-  // CUDA events on the context's stream (median).  Results of the path do not depend on
-  // the choice: the deposit sums are exact integers, and both column-pass forms run the
-  // same radix stages.
+  // CUDA events on the context's stream (median).  The deposit sums are exact integers, the
+  // same for every shape.  Fused and separate x passes, and the two column-pass forms, run the
+  // same radix stages but may round differently in the last bit (from 512^3 on the staged
+  // adjoint z pass applies Green's function once, after its sum).
   int autotune(int reps, pm_tuning* chosen, double* ms_best) override {
     counted_ = false;
     if (reps < 1) reps = 3;
@@ -1593,11 +1598,11 @@ class Engine : public EngineBase {
   // Grid of a particle loop over `work` items of each instance: the blocks that the kernel keeps
   // resident on all SMs, for each instance, or where an instance is no more than kMaxRedBlocks
   // blocks of particles, for the batch; with `sums` always for each instance, so that sums of
-  // doubles are grouped alike in a batch and alone, and their bits the same.  (Several whole waves scatter the blocks in flight over the
-  // lattice as they drift apart: adjoint gather with three waves 112, 769 and 6323 us at 256^3, 512^3
-  // and 1024^3, with one 102, 742 and 5962; forward gather 73, 506 and 4551 with two, 71, 497 and 4470
-  // with one.  One wave over 16 instances of 128^3 mixes their meshes in the L2: adjoint gather
-  // 1204 us against 836 with one each.)
+  // doubles are grouped alike in a batch and alone, and their bits the same.  (Several whole waves
+  // scatter the blocks in flight over the lattice as they drift apart: adjoint gather with three
+  // waves 112, 769 and 6323 us at 256^3, 512^3 and 1024^3, with one 102, 742 and 5962; forward gather
+  // 73, 506 and 4551 with two, 71, 497 and 4470 with one.  One wave over 16 instances of 128^3 mixes
+  // their meshes in the L2: adjoint gather 1204 us against 836 with one each.)
   int wave_grid(const void* fn, long long work, bool sums = false) const {
     const long long need = (work + kPtclThreads - 1) / kPtclThreads;
     int occ = 0;
@@ -1639,7 +1644,7 @@ class Engine : public EngineBase {
   BinGeo bg1_{}, bg4_{};
   BinGeo bgf1_{}, bgf4_{};   // whole-row tiles of the deposit fused with the R2C x pass
   bool fused1_ = false, fused4_ = false;
-  double fused_ms_[4] = {};   // autotuner: separate and fused deposit times (density, density + pi)   // forward (density) / adjoint (density + pi) deposit fused
+  double fused_ms_[4] = {};   // autotuner: separate and fused deposit times (density, density + pi)
   bool counted_ = false;   // the last gather counted the bins of the next deposit
   pm_tuning tune_{};
   pm_tuning tune0_{};            // the default shapes

@@ -2,8 +2,9 @@
 // real type.  Included once per precision.
 //
 //  k_scatter        CIC mass (and adjoint pi) assignment, Sec. 2.2 Eq. 10, int64 fixed point
-//                   with global atomics (the allocation-free density entry point; the
-//                   engine assigns by mesh tiles, bin_kernels.cuh)
+//                   with global atomics (the allocation-free density entry point, deposits
+//                   of few particles and interpolated densities; otherwise the engine
+//                   assigns by mesh tiles, bin_kernels.cuh)
 //  k_gather_fwd     CIC force gather + kick / kick / drift of Eq. 16 (one launch per step);
 //                   counts the deposit bins of the new positions for the next step
 //  k_gather_adj     CIC gather of a and alpha (Eq. 49 F line) + reverse kicks and drift of
